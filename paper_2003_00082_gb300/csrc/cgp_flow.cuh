@@ -1,0 +1,1098 @@
+// The resident solvers' iterations in dataflow form: no grid barrier and no
+// memory fence inside the loop.
+//
+// A block needs two things from the others every iteration: the totals of the
+// three dot products, and w = K u of the rows its product reads (its halo).
+// Both travel in words that show by themselves whether they are the ones
+// waited for, so a reader polls exactly the data it will use:
+//   - every block owns one 128-byte line per bank (two banks by parity) and
+//     stores its partial sums there as one record: FP64 four 64-bit words, each
+//     tagged (fx::pack_record), FP32 one tagged 128-bit word;
+//   - w of a row that another block reads is stored with the reduction's
+//     number in one 128-bit (FP64) or 64-bit (FP32) word.
+// The halo rows' r and s are not published at all: a reader keeps copies of
+// them (ghost rows) and applies the owner's own operations to them every
+// iteration, so both hold the same bits.
+//
+// A bank is rewritten two reductions later.  A block stores its sums of
+// reduction k + 1 only after it has read all it needs of reduction k (the
+// stored sums depend on what it read), and reduction k + 2's words only after
+// it has seen every block's sums of k + 1, so no word is overwritten before
+// its readers have it.
+//
+// What bounds it: 152 blocks that exchange one flag each way take 8.1k clocks
+// an exchange through a release/acquire counter, 5.4k through slots 16 bytes
+// apart (the pollers queue on the shared lines), 3.5k through slots on lines
+// of their own stored with release, 2.6k stored relaxed; a line read on the
+// other die just after it was written costs about 1.7k of that.  Polling
+// loads the same network that the words travel on: one 32-byte load per block
+// and round is faster than three 16-byte ones (2.6k against 3.7k clocks from the
+// block barrier to the last share at 512x256).  The rest of
+// an iteration is a chain of short steps (warp sums, block sums, totals,
+// scalars), each of which is written for latency here.
+#pragma once
+
+#include "cgp_solver.cuh"
+
+namespace cgp {
+namespace {
+
+constexpr int kMaxShares = 8;   // groups of blocks whose records are folded by one warp each
+
+// This block's line of bank (red & 1).
+__device__ __forceinline__ unsigned char* flow_line(const Desc& d, int red, int blk) {
+  return reinterpret_cast<unsigned char*>(d.tpart) + ((size_t)blk * 2 + (red & 1)) * kLineBytes;
+}
+
+// Limit of a polling loop: d.spin_ns of wall-clock time, or as soon as another
+// block has given up.
+struct PollLimit {
+  int* timeout;
+  long long spin_ns;
+  unsigned long long t0 = 0;
+  unsigned spins = 0;
+  __device__ PollLimit(const Desc& d) : timeout(&d.res->timeout), spin_ns(d.spin_ns) {}
+  __device__ bool expired() {
+    if ((++spins & 63u) != 0) return false;
+    if (*(volatile int*)timeout) return true;
+    const unsigned long long now = global_ns();
+    if (t0 == 0) {
+      t0 = now;
+    } else if ((long long)(now - t0) > spin_ns) {
+      atomicExch(timeout, 1);
+      return true;
+    }
+    return false;
+  }
+};
+
+// Groups the blocks of a solve are polled in (32 blocks a pass each) by at most
+// `most` warps.
+__device__ __forceinline__ int flow_groups(int nblk, int most) {
+  return min(min((nblk + 31) / 32, most), kMaxShares);
+}
+
+// Row il's product with columns and values in shared memory (columns renumbered
+// into ext), its entries taken eight at a time with their loads issued together
+// (a row of a triangular mesh has about seven).
+template <typename V>
+__device__ __forceinline__ V row_product(const int* __restrict__ col, const V* __restrict__ val, const V* ext, int k0,
+                                         int k1) {
+  constexpr int B = 8;
+  V s = V(0);
+  for (int k = k0; k < k1; k += B) {
+    int c[B];
+    V a[B];
+#pragma unroll
+    for (int q = 0; q < B; ++q) c[q] = k + q < k1 ? col[k + q] : 0;
+#pragma unroll
+    for (int q = 0; q < B; ++q) a[q] = k + q < k1 ? val[k + q] : V(0);
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      const V u = ext[c[q]];
+      if (k + q < k1) s = fma(a[q], u, s);
+    }
+  }
+  return s;
+}
+
+// Rows below nloc of the calling thread among nt threads, T lanes per row.
+template <int T, typename V, typename Op>
+__device__ __forceinline__ void flow_rows(const int* __restrict__ row, const int* __restrict__ col,
+                                          const V* __restrict__ val, const V* ext, int nloc, int t, int nt, Op op) {
+  if constexpr (T == 1) {
+    for (int il = t; il < nloc; il += nt) op(il, row_product(col, val, ext, row[il], row[il + 1]));
+  } else {
+    const int g = t / T, l = t % T, ng = nt / T;
+    for (int base = 0; base < nloc; base += ng) {
+      const int il = base + g;
+      V s = V(0);
+      if (il < nloc) {
+        const int k1 = row[il + 1];
+        for (int k = row[il] + l; k < k1; k += T) s = fma(val[k], ext[col[k]], s);
+      }
+#pragma unroll
+      for (int o = T / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, T);
+      if (il < nloc && l == 0) op(il, s);
+    }
+  }
+}
+
+// ---- FP64 -------------------------------------------------------------------
+
+__device__ __forceinline__ void st_relaxed_v4(void* p, const uint64_t (&w)[4]) {
+  asm volatile("st.relaxed.gpu.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(w[0]), "l"(w[1]), "l"(w[2]),
+               "l"(w[3])
+               : "memory");
+}
+__device__ __forceinline__ void ld_relaxed_v4(const void* p, uint64_t (&w)[4]) {
+  asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(w[0]), "=l"(w[1]), "=l"(w[2]), "=l"(w[3])
+               : "l"(p)
+               : "memory");
+}
+
+// The block's partial sums of three per-thread values, stored as its record of
+// reduction `red`.  Images as in put_partials64: exact up to the truncation of
+// each term 2^-54 below the largest one of its warp or block.  Only the first
+// `act` warps have rows; after the block barrier inside, warps fw .. fw + 2 fold
+// a component each and warp fw stores the record.
+__device__ __forceinline__ void flow_put(const Desc& d, int lb, int red, int act, int fw, const double (&v)[3],
+                                         Shared& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < act) {
+    int E[3];
+    long long S[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) E[c] = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx64_exponent(v[c]));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) S[c] = warp_sum57(E[c] < fx::kBadExp ? fx64_image(v[c], E[c]) : 0ll);
+    if (lane < 3) {
+      sh.whi[lane][warp] = lane == 0 ? S[0] : (lane == 1 ? S[1] : S[2]);
+      sh.wexp[lane][warp] = lane == 0 ? E[0] : (lane == 1 ? E[1] : E[2]);
+    }
+  }
+  if (threadIdx.x == 0) sh.tflag = 1;
+  __syncthreads();
+  const int c = warp - fw;
+  if (c >= 0 && c < 3) {
+    const long long sw = lane < act ? sh.whi[c][lane] : 0ll;
+    const int ew = lane < act ? sh.wexp[c][lane] : 1;
+    const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)ew);
+    const long long S = warp_sum57(E < fx::kBadExp ? (sw >> min(E - ew + 5, 63)) : 0ll);
+    if (lane == 0) {
+      sh.bsum[c] = S;
+      sh.bexp[c] = E;
+    }
+    named_sync(2, 96);
+    if (c == 0 && lane == 0) {
+      const int64_t Sa[3] = {S, sh.bsum[1], sh.bsum[2]};
+      const int Ea[3] = {E, sh.bexp[1], sh.bexp[2]};
+      uint64_t w[4];
+      fx::pack_record(Sa, Ea, red, w);
+      st_relaxed_v4(flow_line(d, red, lb), w);
+    }
+  }
+}
+
+// Polling warp q < G: wait for the records of the blocks 32 q + lane (+ 32 G
+// ...) of reduction `red`; the warp's share of the totals goes to
+// sh.phi/pexp[c][q], value phi 2^(pexp - 1074), |phi| < 2^62.  A block's
+// partial enters with 57 bits relative to the largest one.  False (on every
+// lane) when the wait gave up.
+__device__ __forceinline__ bool flow_poll(const Desc& d, int red, int q, int G, Shared& sh) {
+  const int lane = threadIdx.x & 31;
+  PollLimit lim(d);
+  const uint64_t tag = fx::record_tag(red);
+  long long acc[3] = {0, 0, 0};
+  int Ea[3] = {1, 1, 1};
+  for (int base = 32 * q; base < d.nblk; base += 32 * G) {
+    const int j = base + lane;
+    uint64_t w[4];
+    const void* line = flow_line(d, red, j < d.nblk ? j : base);
+    while (true) {
+      ld_relaxed_v4(line, w);
+      if (__all_sync(0xffffffffu, fx::record_current(w, tag))) break;
+      if (__any_sync(0xffffffffu, lim.expired())) return false;
+    }
+    int E[3];
+    long long S[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int e = j < d.nblk ? fx::record_exponent(w, c) : 1;
+      S[c] = j < d.nblk ? (long long)fx::record_mantissa(w, c) : 0ll;
+      E[c] = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+      S[c] = E[c] < fx::kBadExp ? (S[c] >> min(E[c] - e + 5, 63)) : 0ll;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const long long t = warp_sum57(S[c]);
+      if (base == 32 * q) {
+        acc[c] = t;
+        Ea[c] = E[c] + 5;
+      } else {   // |acc|, |t| < 2^62: one more bit
+        const int F = max(Ea[c], E[c] + 5);
+        acc[c] = ((acc[c] >> min(F - Ea[c], 63)) + (t >> min(F - (E[c] + 5), 63))) >> 1;
+        Ea[c] = F + 1;
+      }
+    }
+  }
+  if (lane < 3) {
+    sh.phi[lane][q] = lane == 0 ? acc[0] : (lane == 1 ? acc[1] : acc[2]);
+    sh.pexp[lane][q] = lane == 0 ? Ea[0] : (lane == 1 ? Ea[1] : Ea[2]);
+  }
+  return true;
+}
+
+// Nearest double of X 2^(E - 1074), |X| < 2^62: one conversion and an integer
+// add to its exponent where the result is a normal number.
+__device__ __forceinline__ double scaled_double(long long X, int E) {
+  const double y = (double)X;
+  const int e = (int)((fx::dbits(y) >> 52) & 0x7FF) + E - 1074;
+  if (X != 0 && e > 0 && e < 0x7FF) return fx::from_bits(fx::dbits(y) + ((uint64_t)(int64_t)(E - 1074) << 52));
+  return fx::to_double((fx::I128)X, E >= fx::kBadExp ? E : E + kSlot64Shift);   // NaN for a non-finite term
+}
+
+// A reciprocal of a normal a to about 22 bits, its exponent set by integer
+// operations so that any exponent moderate() accepts is safe.
+__device__ __forceinline__ double reciprocal_seed(double a) {
+  const unsigned long long b = fx::dbits(a);
+  const float m = __uint_as_float(0x3F800000u | (unsigned)((b >> 29) & 0x7FFFFFull));   // [1, 2)
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));                                 // [0.5, 1]
+  const unsigned f = __float_as_uint(r);
+  const int e = (int)(f >> 23) - 127 + 2046 - (int)((b >> 52) & 0x7FF);
+  return fx::from_bits(((unsigned long long)e << 52) | ((unsigned long long)(f & 0x7FFFFFu) << 29));
+}
+__device__ __forceinline__ bool moderate(double a) {   // a positive normal with room to spare on both sides
+  const int e = __double2hiint(a) >> 20;
+  return e > 64 && e < 1982;
+}
+
+// One warp: the totals of the shares and the scalars of the next update.  An
+// FP64 operation takes 64 clocks from issue to use whatever the number of
+// active lanes, and the compiler's division about nine of them in a chain (564
+// clocks), so the lanes share the work: lane 0 forms the quotient alpha by one
+// residual correction (Markstein's) with the reciprocal that lane 1 refines
+// meanwhile by one Newton step, while lane 2 refines 1 / gamma for the next
+// iteration: three operations after the denominator.
+//   beta = gamma / gamma_old, alpha = gamma / (delta - beta gamma / alpha_old);
+// ab[k & 1] alpha and beta (two copies: the update of p and x still reads the
+// last ones), sc[4] the stop bound, sc[5] (r,r), isc[0] the stop status.
+// Keeps inv[0] = 1 / gamma_old and inv[1] = 1 / (gamma_old alpha_old); returns
+// what flow_scalars_rest needs to form the next ones off the critical path.
+struct ScalarRest {
+  double t, e, den;
+};
+__device__ __forceinline__ ScalarRest flow_scalars(int G, int k, bool last, const double (&inv)[2], Shared& sh) {
+  const int lane = threadIdx.x & 31;
+  int E[3];
+  long long X[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    X[c] = lane < G ? sh.phi[c][lane] : 0ll;
+    const int e = lane < G ? sh.pexp[c][lane] : 1;
+    E[c] = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+    X[c] = E[c] < fx::kBadExp ? (X[c] >> min(E[c] - e + 3, 63)) : 0ll;   // eight shares of 59 bits
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) X[c] = warp_sum57(X[c]);
+  const double v = scaled_double(lane == 1 ? X[1] : (lane == 2 ? X[2] : X[0]),
+                                 (lane == 1 ? E[1] : (lane == 2 ? E[2] : E[0])) + 3);
+  const double g = __shfl_sync(0xffffffffu, v, 0), dl = __shfl_sync(0xffffffffu, v, 1);
+  double beta = 0.0, den = dl;
+  if (k > 0) {
+    const double m = (lane == 0 ? -g : g) * (lane == 0 ? g : inv[0]);   // lane 0: -gamma^2; others: beta
+    den = __shfl_sync(0xffffffffu, fma(m, inv[1], dl), 0);
+    beta = __shfl_sync(0xffffffffu, m, 1);
+  }
+  const double rr = __shfl_sync(0xffffffffu, v, 2);
+  ScalarRest q;
+  q.den = den;
+  double alpha;
+  int st = -1;
+  if (moderate(den) && moderate(g)) {
+    const double a = lane == 2 ? g : den;
+    const double y0 = reciprocal_seed(a);
+    const double t1 = fma(lane == 0 ? g : -a, y0, lane == 0 ? 0.0 : 1.0);          // q0; 1 - a y0
+    if (!finite_bits(rr)) st = CGP_ERR_NONFINITE;
+    else if (nonneg_le(rr, sh.sc[4])) st = CGP_OK;   // (r,r) and (tol |b|)^2 are >= 0
+    else if (last) st = CGP_ERR_NOT_CONVERGED;
+    q.t = fma(lane == 0 ? -den : t1, lane == 0 ? t1 : y0, lane == 0 ? g : y0);     // g - den q0; y1
+    const double y1 = __shfl_sync(0xffffffffu, q.t, 1);
+    q.e = fma(lane == 0 ? q.t : -a, lane == 0 ? y1 : q.t, lane == 0 ? t1 : 1.0);   // alpha; 1 - a y1
+    alpha = q.e;
+  } else {
+    if (!finite_bits(g) || !finite_bits(dl) || !finite_bits(rr)) st = CGP_ERR_NONFINITE;
+    else if (nonneg_le(rr, sh.sc[4])) st = CGP_OK;
+    else if (last) st = CGP_ERR_NOT_CONVERGED;
+    alpha = g / den;
+    q.t = 1.0 / g;
+    q.e = 0.0;
+  }
+  if (lane == 0) {
+    if (st < 0 && !(positive_bits(g) && positive_bits(alpha) && finite_bits(alpha))) st = CGP_ERR_BREAKDOWN;
+    sh.isc[0] = st;
+    sh.ab[k & 1][0] = alpha;
+    sh.ab[k & 1][1] = beta;
+    sh.sc[5] = rr;
+  }
+  return q;
+}
+// 1 / gamma (lane 2) and 1 / (gamma alpha) = den / gamma^2 on every lane.
+__device__ __forceinline__ void flow_scalars_rest(const ScalarRest& q, double (&inv)[2]) {
+  inv[0] = __shfl_sync(0xffffffffu, fma(q.e, q.t, q.t), 2);
+  inv[1] = q.den * inv[0] * inv[0];
+}
+
+// Word of row j's w in the publication of reduction `red`.
+__device__ __forceinline__ ulonglong2* flow_w64(const Desc& d, int red, int j) {
+  return reinterpret_cast<ulonglong2*>(d.pub64) + (size_t)(red & 1) * d.n + j;
+}
+
+// FP64 Jacobi-PCG in the single-reduction form (solve_fp64_sr describes the
+// recurrences) with rows resident in shared memory and dataflow iterations.
+// The passes around the loop (projections, true residual) use the group
+// barrier.
+//
+// Roles (a block has at least eight warps): the first half (ct threads) holds
+// the rows; four warps with an operation always ready fill the FP64 pipe, so
+// eight lose nothing in the product and halve the integer work of the partial
+// sums.  The other half folds and stores the partial sums, fetches the halo's
+// w, polls, derives the scalars and updates the ghost rows.  Keeping the rows'
+// r, s, w, u in registers (four rows a thread) was slower: 7.4 us an iteration.
+//
+// Measured at 512x256 on 152 blocks in O-grid tiles: 6.83 us an iteration with
+// the counter barrier and slots 16 bytes apart, 6.34 us in this form.  About
+// 4.5k of its 13.1k clocks are the product and the dot products on the FP64 pipe,
+// 1.3k the recurrences, 2.5k the exchange up to the last share, 1.7k the scalars.
+constexpr int kFlowMinBlock = 256;
+template <int T>
+__device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  const int tid = threadIdx.x, bd = blockDim.x, warp = tid >> 5, nw = bd >> 5;
+  const int chunk = (d.n + d.nblk - 1) / d.nblk;
+  const int r0 = min(d.n, lb * chunk), r1 = min(d.n, r0 + chunk), nloc = r1 - r0;
+  const size_t n = d.n;
+  Group grp{d.bar, &d.res->timeout, (unsigned)d.nblk, 0u, d.spin_ns};
+  int red = 0;
+  const int ow = nw / 2, ct = 32 * ow;                  // warps and threads with rows
+  const int act = min(ow, (nloc * T + 31) / 32);        // of those, warps that have any
+  const int G = flow_groups(d.nblk, nw - ow);           // warps ow .. ow + G - 1 poll
+  double* const R0 = d.pub64 + 4 * n;                // r of a pass's start, for the ghost rows
+  int* const mark = reinterpret_cast<int*>(d.z);     // rows that another block reads
+
+  // shared memory: own vectors, the product's input (CSR: own rows and halo;
+  // stencil: the padded box), D^-1 and ghost r, s, w of the halo, the system,
+  // its indices, and one byte per own row (published or not)
+  const bool st = d.stencil;
+  double* base = reinterpret_cast<double*>(dsm);
+  double* x = base;
+  double* r = base + chunk;
+  double* ua = base + 2 * chunk;     // u_k and u_(k+1) alternate
+  double* ub = base + 3 * chunk;
+  double* w = base + 4 * chunk;
+  double* p = base + 5 * chunk;
+  double* s = base + 6 * chunk;
+  double* di = base + 7 * chunk;
+  double* bp = base + 8 * chunk;
+  double* ext = base + 9 * chunk;
+  double* dih = ext + (st ? d.box_cap : chunk + d.halo_cap);
+  double* val = dih + d.halo_cap;                    // CSR: [nnz_cap]; stencil: [7][chunk] planes
+  double* gr = val + (st ? 7 * chunk : d.res_nnz_cap);
+  double* gs = gr + d.halo_cap;
+  double* gw = gs + d.halo_cap;
+  int* row = reinterpret_cast<int*>(gw + d.halo_cap);   // CSR: offsets [chunk + 1]; stencil: box positions [chunk]
+  int* col = row + chunk + 1;
+  int* hid = st ? row + chunk : col + d.res_nnz_cap;    // global row of each halo entry
+  int* hpos = hid + d.halo_cap;                         // stencil: its box position
+  unsigned char* pub = reinterpret_cast<unsigned char*>(st ? hpos + d.halo_cap : hid + d.halo_cap);
+  const int h0 = d.hptr[lb], nh = d.hptr[lb + 1] - h0;
+  int Ba = 0;
+  if (st) {
+    Ba = d.bdim[lb];
+    for (int q = tid; q < d.box_cap; q += bd) ext[q] = 0.0;   // the ring outside the domain stays zero
+    for (int k = 0; k < 7; ++k)
+      for (int i = tid; i < nloc; i += bd) val[k * chunk + i] = d.planes[(size_t)k * n + r0 + i];
+    for (int i = tid; i < nloc; i += bd) row[i] = d.bpos[r0 + i];
+    for (int h = tid; h < nh; h += bd) hpos[h] = d.hpos[h0 + h];
+  } else {
+    const int k0 = nloc > 0 ? d.rowptr[r0] : 0;
+    const int nnzl = nloc > 0 ? d.rowptr[r1] - k0 : 0;
+    for (int i = tid; i <= nloc; i += bd) row[i] = d.rowptr[r0 + i] - k0;
+    for (int k = tid; k < nnzl; k += bd) {
+      col[k] = d.lcol[k0 + k];
+      val[k] = d.val[k0 + k];
+    }
+  }
+  for (int h = tid; h < nh; h += bd) {
+    const int j = d.hidx[h0 + h];
+    hid[h] = j;
+    dih[h] = d.dinv[j];
+  }
+  for (int i = tid; i < nloc; i += bd) di[i] = d.dinv[r0 + i];
+
+  auto own_at = [&](int i) { return st ? row[i] : i; };
+  auto halo_at = [&](int h) { return st ? hpos[h] : nloc + h; };
+  // the product's rows of thread t among nt
+  auto rows = [&](int t, int nt, auto op) {
+    if (st) spmv_box(row, val, chunk, ext, Ba, nloc, t, nt, op);
+    else flow_rows<T>(row, col, val, ext, nloc, t, nt, op);
+  };
+  // this block's words start empty, its rows unmarked; the barrier of the first
+  // reduction orders that before any block polls or marks
+  if (tid < 2) {
+    const uint64_t none[4] = {0, 0, 0, 0};
+    st_relaxed_v4(flow_line(d, tid, lb), none);
+  }
+  for (int i = tid; i < nloc; i += bd) {
+    *flow_w64(d, 0, r0 + i) = make_ulonglong2(0ull, 0ull);
+    *flow_w64(d, 1, r0 + i) = make_ulonglong2(0ull, 0ull);
+    mark[r0 + i] = 0;
+  }
+  // ---- means of b and x0 ----
+  {
+    double v2[2] = {0.0, 0.0};
+    for (int i = tid; i < nloc; i += bd) {
+      v2[0] += d.b[r0 + i];
+      if (d.use_x0) v2[1] += d.x[r0 + i];
+    }
+    put_partials<2>(d, lb, red, v2, sh);
+    if (!grp.sync(sh)) return;
+    get_totals<2>(d, red, sh);
+    ++red;
+  }
+  for (int h = tid; h < nh; h += bd) mark[hid[h]] = 1;
+  // ---- projected b and x0; x0 published for the first product ----
+  {
+    const double mb = d.fixed ? 0.0 : sh.tot[0] / d.n, mx = d.fixed ? 0.0 : sh.tot[1] / d.n;
+    double v1[1] = {0.0};
+    for (int i = tid; i < nloc; i += bd) {
+      const double bi = is_fixed(d, r0 + i) ? 0.0 : d.b[r0 + i] - mb;
+      bp[i] = bi;
+      v1[0] += bi * bi;
+      const double xi = (d.use_x0 && !is_fixed(d, r0 + i)) ? d.x[r0 + i] - mx : 0.0;
+      x[i] = xi;
+      d.x[r0 + i] = xi;
+    }
+    put_partials<1>(d, lb, red, v1, sh);
+    if (!grp.sync(sh)) return;
+    get_totals<1>(d, red, sh);
+    ++red;
+  }
+  for (int i = tid; i < nloc; i += bd) pub[i] = (unsigned char)__ldcg(mark + r0 + i);
+  const double bnorm = sqrt(sh.tot[0]);
+  if (!isfinite(bnorm)) { finish(d, lb, CGP_ERR_NONFINITE, 0, 0, 0.0, 0.0, bnorm); return; }
+  if (bnorm == 0.0) {
+    for (int i = tid; i < nloc; i += bd) d.x[r0 + i] = 0.0;
+    finish(d, lb, CGP_OK, 0, 0, 0.0, 0.0, 0.0);
+    return;
+  }
+  const double stop = d.tol * bnorm, stop2 = stop * stop;
+  if (tid == 0) sh.sc[4] = stop2;   // the test ||r||^2 <= (tol ||b||)^2 needs no square root
+
+  int its = 0, restarts = 0, status = CGP_ERR_NOT_CONVERGED, pending = -1;
+  double rr_rec = 0.0, rr_true = 0.0;
+  bool first = true;
+  while (true) {
+    // ---- true residual of the projected, published x: r = bp - K x, u = D^-1 r; r published ----
+    {
+      double v1[1] = {0.0};
+      for (int i = tid; i < nloc; i += bd) ext[own_at(i)] = x[i];
+      for (int h = tid; h < nh; h += bd) ext[halo_at(h)] = __ldcg(d.x + hid[h]);
+      __syncthreads();
+      rows(tid, bd, [&](int il, double sum) {
+        const double t = bp[il] - sum;
+        r[il] = t;
+        ua[il] = di[il] * t;
+        R0[r0 + il] = t;
+        v1[0] += t * t;
+      });
+      put_partials<1>(d, lb, red, v1, sh);
+      if (!grp.sync(sh)) return;   // also publishes r for the ghost rows
+      get_totals<1>(d, red, sh);
+      ++red;
+    }
+    rr_true = sh.tot[0];
+    if (first) rr_rec = rr_true;
+    if (!isfinite(rr_true)) { status = CGP_ERR_NONFINITE; break; }
+    if (rr_true <= stop2) { status = CGP_OK; break; }
+    if (pending >= 0) { status = pending; break; }
+    if (its >= d.max_it || restarts >= kMaxRestarts) { status = CGP_ERR_NOT_CONVERGED; break; }
+    if (!first) ++restarts;
+    first = false;
+
+    // ---- u_0 and the ghost rows; then iterations from the product w_0 = K u_0 ----
+    for (int i = tid; i < nloc; i += bd) ext[own_at(i)] = ua[i];
+    for (int h = tid; h < nh; h += bd) {
+      const double rj = __ldcg(R0 + hid[h]);
+      gr[h] = rj;
+      ext[halo_at(h)] = dih[h] * rj;
+    }
+    int k = 0;                           // products formed in this pass, less one
+    double inv[2] = {0.0, 0.0};          // the scalars' reciprocals (warp ow)
+    while (true) {
+      double* const uc = (k & 1) ? ub : ua;   // u_k
+      double* const up = (k & 1) ? ua : ub;   // u_(k-1), then u_(k+1)
+      __syncthreads();
+      // ---- w_k = K u_k, published where another block reads it; the partial sums ----
+      double v3[3] = {0.0, 0.0, 0.0};
+      const unsigned long long tag = (unsigned long long)red + 1;
+      if (tid < ct) {
+        rows(tid, ct, [&](int il, double sum) {
+          const double ui = uc[il], ri = r[il];
+          const bool out = pub[il];
+          w[il] = sum;
+          v3[0] = fma(ri, ui, v3[0]);
+          v3[1] = fma(sum, ui, v3[1]);
+          v3[2] = fma(ri, ri, v3[2]);
+          if (out) st_relaxed_b128(flow_w64(d, red, r0 + il), fx::dbits(sum), tag);
+        });
+      }
+      flow_put(d, lb, red, act, ow, v3, sh);
+      // ---- p_(k-1) = u_(k-1) + beta p_(k-2), x += alpha p_(k-1) while the words travel ----
+      if (k > 0 && tid < ct) {
+        const double alpha = sh.ab[(k - 1) & 1][0], beta = sh.ab[(k - 1) & 1][1];
+        for (int i = tid; i < nloc; i += ct) {
+          const double pi = k == 1 ? up[i] : fma(beta, p[i], up[i]);
+          p[i] = pi;
+          x[i] = fma(alpha, pi, x[i]);
+        }
+      }
+      // ---- the halo's w, then the records ----
+      ScalarRest rest;
+      if (warp >= ow) {
+        PollLimit lim(d);
+        constexpr int B = 4;   // loads of a thread in flight
+        const int nt = bd - ct;
+        for (int h = bd - 1 - tid; h < nh; h += B * nt) {   // the last warps first: they do not poll
+          ulonglong2 a[B];
+#pragma unroll
+          for (int q = 0; q < B; ++q)
+            a[q] = h + q * nt < nh ? ld_relaxed_b128(flow_w64(d, red, hid[h + q * nt])) : make_ulonglong2(0ull, tag);
+#pragma unroll
+          for (int q = 0; q < B; ++q) {
+            while (a[q].y != tag && !lim.expired()) a[q] = ld_relaxed_b128(flow_w64(d, red, hid[h + q * nt]));
+            if (a[q].y != tag) sh.tflag = 0;
+            if (h + q * nt < nh) gw[h + q * nt] = fx::from_bits(a[q].x);
+          }
+        }
+        if (warp < ow + G) {
+          if (!flow_poll(d, red, warp - ow, G, sh)) sh.tflag = 0;
+          named_sync(1, 32 * G);
+          if (warp == ow) rest = flow_scalars(G, k, its + k >= d.max_it, inv, sh);
+        }
+      }
+      __syncthreads();
+      if (!sh.tflag) return;
+      ++red;
+      const int stop_st = sh.isc[0];
+      if (stop_st >= 0) {
+        if (stop_st != CGP_OK) pending = stop_st;
+        break;
+      }
+      const double alpha = sh.ab[k & 1][0], beta = sh.ab[k & 1][1];
+      // ---- own rows and ghost rows: s, r, u_(k+1) ----
+      if (tid < ct) {
+        for (int i = tid; i < nloc; i += ct) {
+          const double si = k == 0 ? w[i] : fma(beta, s[i], w[i]);
+          s[i] = si;
+          const double ri = fma(-alpha, si, r[i]);
+          r[i] = ri;
+          const double ui = di[i] * ri;
+          up[i] = ui;
+          ext[own_at(i)] = ui;
+        }
+      } else {
+        for (int h = bd - 1 - tid; h < nh; h += bd - ct) {
+          const double sj = k == 0 ? gw[h] : fma(beta, gs[h], gw[h]);
+          gs[h] = sj;
+          const double rj = fma(-alpha, sj, gr[h]);
+          gr[h] = rj;
+          ext[halo_at(h)] = dih[h] * rj;
+        }
+        if (warp == ow) flow_scalars_rest(rest, inv);
+      }
+      ++k;
+    }
+    its += k;
+    rr_rec = sh.sc[5];
+    // ---- x -= mean(x), published for the true residual ----
+    {
+      double v1[1] = {0.0};
+      for (int i = tid; i < nloc; i += bd) v1[0] += x[i];
+      put_partials<1>(d, lb, red, v1, sh);
+      if (!grp.sync(sh)) return;
+      get_totals<1>(d, red, sh);
+      ++red;
+    }
+    const double mxf = d.fixed ? 0.0 : sh.tot[0] / d.n;
+    for (int i = tid; i < nloc; i += bd) {
+      const double xi = x[i] - mxf;
+      x[i] = xi;
+      d.x[r0 + i] = xi;
+    }
+    if (!grp.sync(sh)) return;
+  }
+  finish(d, lb, status, its, restarts, sqrt(rr_rec) / bnorm, sqrt(rr_true) / bnorm, bnorm);
+}
+
+// ---- FP32 (the inner iterations of MIXED) -----------------------------------
+
+// The block's partial sums of three per-thread values as its word of reduction
+// `red`: {v0, v1, v2, red + 1}.
+__device__ __forceinline__ void flow_put_f(const Desc& d, int lb, int red, int act, const float (&v)[3], Shared& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < act) {
+    float t[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) t[c] = warp_sum(v[c]);
+    if (lane < 3) sh.fred[lane][warp] = lane == 0 ? t[0] : (lane == 1 ? t[1] : t[2]);
+  }
+  if (threadIdx.x == 0) sh.tflag = 1;
+  __syncthreads();
+  if (warp == 0) {
+    float t[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      t[c] = lane < act ? sh.fred[c][lane] : 0.0f;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) t[c] += __shfl_xor_sync(0xffffffffu, t[c], o);   // at most 16 warps
+    }
+    if (lane == 0)
+      st_relaxed_b128(flow_line(d, red, lb),
+                      ((unsigned long long)__float_as_uint(t[1]) << 32) | __float_as_uint(t[0]),
+                      ((unsigned long long)(unsigned)(red + 1) << 32) | __float_as_uint(t[2]));
+  }
+}
+
+// Warp q < G: wait for the words of the blocks 32 q + lane (+ 32 G ...); the
+// warp's share of the totals goes to sh.pf[c][q] (fixed order: the same bits
+// in every block).
+__device__ __forceinline__ bool flow_poll_f(const Desc& d, int red, int q, int G, Shared& sh) {
+  const int lane = threadIdx.x & 31;
+  PollLimit lim(d);
+  const unsigned tag = (unsigned)(red + 1);
+  float acc[3] = {0.0f, 0.0f, 0.0f};
+  for (int base = 32 * q; base < d.nblk; base += 32 * G) {
+    const int j = base + lane;
+    const void* line = flow_line(d, red, j < d.nblk ? j : base);
+    ulonglong2 a;
+    while (true) {
+      a = ld_relaxed_b128(line);
+      if (__all_sync(0xffffffffu, (unsigned)(a.y >> 32) == tag)) break;
+      if (__any_sync(0xffffffffu, lim.expired())) return false;
+    }
+    if (j < d.nblk) {
+      acc[0] += __uint_as_float((unsigned)a.x);
+      acc[1] += __uint_as_float((unsigned)(a.x >> 32));
+      acc[2] += __uint_as_float((unsigned)a.y);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) acc[c] = warp_sum(acc[c]);
+  if (lane < 3) sh.pf[lane][q] = lane == 0 ? acc[0] : (lane == 1 ? acc[1] : acc[2]);
+  return true;
+}
+
+__device__ __forceinline__ bool finite_bits(float x) { return ((__float_as_uint(x) >> 23) & 0xFFu) != 0xFFu; }
+
+// One warp: the totals and the scalars of the next FP32 update: abf[k & 1]
+// alpha and beta, fsc[3] ||r_0||^2 of the sweep, fsc[4] and fsc[5] the stop
+// bounds, isc[0] the stop flag (0: stop, 1: non-finite, 2: breakdown); gamma
+// and alpha of the last iteration stay with the warp in old[].
+__device__ __forceinline__ void flow_scalars_f(int G, int k, bool last, float (&old)[2], Shared& sh) {
+  const int lane = threadIdx.x & 31, c = lane >> 3, q = lane & 7;
+  float v = c < 3 && q < G ? sh.pf[c][q] : 0.0f;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  const float g = __shfl_sync(0xffffffffu, v, 0), dl = __shfl_sync(0xffffffffu, v, 8);
+  const float rr = __shfl_sync(0xffffffffu, v, 16);
+  float beta = 0.0f, den = dl;
+  if (k > 0) {   // two quotients of known terms side by side, then the one that needs the totals' difference
+    beta = g / old[0];
+    den = dl - beta * (g / old[1]);
+  }
+  const float alpha = g / den;
+  const float rr0 = k == 0 ? rr : sh.fsc[3];
+  int st = -1;
+  if (!finite_bits(rr) || !finite_bits(g) || !finite_bits(dl)) st = 1;
+  else if (rr <= fmaxf(sh.fsc[4] * rr0, sh.fsc[5])) st = 0;   // inner tolerance reached
+  else if (last) st = 0;
+  if (st < 0 && !(g > 0.0f && alpha > 0.0f && finite_bits(alpha))) st = 2;
+  __syncwarp();
+  if (lane == 0) {
+    if (k == 0) sh.fsc[3] = rr;
+    sh.isc[0] = st;
+    sh.abf[k & 1][0] = alpha;
+    sh.abf[k & 1][1] = beta;
+  }
+  old[0] = g;
+  old[1] = alpha;
+}
+
+__device__ __forceinline__ unsigned long long* flow_w32(const Desc& d, int red, int j) {
+  return reinterpret_cast<unsigned long long*>(d.f32pub) + (size_t)(red & 1) * d.n + j;
+}
+
+// Mixed precision with rows resident: the FP64 refinement and the FP32 inner
+// recurrences of solve_mixed, the inner iterations in dataflow form.
+//
+// An inner iteration's arithmetic is small; what it costs besides the exchange
+// is shared-memory instructions.  R > 0 (one lane per row, at most R rows a
+// thread) therefore keeps r, s, w, u, D^-1 of a thread's rows and the first
+// eight entries of each (values, 16-bit positions in the product's input) in
+// registers: a row's product is eight independent gathers, and longer rows go
+// on from the shared-memory slice.  R = 0 keeps everything in shared memory.
+// At 512x256 on 152 blocks an inner iteration takes 2.55 us (3.69 us with the
+// counter barrier), at 64x32 on 9 blocks 2.0 us (4.0 us).
+template <int T, int R>
+__device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
+  extern __shared__ __align__(16) unsigned char dsm[];
+  static_assert(R == 0 || T == 1, "register rows take one lane each");
+  constexpr int NR = R > 0 ? R : 1;
+  constexpr int NE = 8;                              // entries of a row in registers
+  const int tid = threadIdx.x, bd = blockDim.x, warp = tid >> 5, nw = bd >> 5;
+  const int chunk = (d.n + d.nblk - 1) / d.nblk;
+  const int r0 = min(d.n, lb * chunk), r1 = min(d.n, r0 + chunk), nloc = r1 - r0;
+  const size_t n = d.n;
+  Group grp{d.bar, &d.res->timeout, (unsigned)d.nblk, 0u, d.spin_ns};
+  int red = 0;
+  const int act = min(nw, (nloc * T + 31) / 32);     // warps with rows
+  const int G = flow_groups(d.nblk, nw);
+  const int f0 = G < nw ? 32 * G : 0;                // threads from here on fetch the halo's w
+  float* const R0 = d.f32pub + 4 * n;                // r of a sweep's start, for the ghost rows
+  int* const mark = reinterpret_cast<int*>(d.z);     // rows that another block reads
+
+  float* f = reinterpret_cast<float*>(dsm);
+  float* ir = f;
+  float* iu = f + chunk;
+  float* iw = f + 2 * chunk;
+  float* ip = f + 3 * chunk;
+  float* is = f + 4 * chunk;
+  float* ie = f + 5 * chunk;
+  float* di = f + 6 * chunk;
+  float* ext = f + 7 * chunk;                   // [chunk + halo_cap]
+  float* dih = ext + chunk + d.halo_cap;        // [halo_cap]
+  float* val = dih + d.halo_cap;                // [nnz_cap]
+  float* gr = val + d.res_nnz_cap;              // [halo_cap] each: ghost r, s and fetched w
+  float* gs = gr + d.halo_cap;
+  float* gw = gs + d.halo_cap;
+  int* row = reinterpret_cast<int*>(gw + d.halo_cap);
+  int* col = row + chunk + 1;
+  int* hid = col + d.res_nnz_cap;
+  unsigned char* pub = reinterpret_cast<unsigned char*>(hid + d.halo_cap);
+  const int h0 = d.hptr[lb], nh = d.hptr[lb + 1] - h0;
+  {
+    const int k0 = nloc > 0 ? d.rowptr[r0] : 0;
+    const int nnzl = nloc > 0 ? d.rowptr[r1] - k0 : 0;
+    for (int i = tid; i <= nloc; i += bd) row[i] = d.rowptr[r0 + i] - k0;
+    for (int k = tid; k < nnzl; k += bd) {
+      col[k] = d.lcol[k0 + k];
+      val[k] = d.val32[k0 + k];
+    }
+    for (int h = tid; h < nh; h += bd) {
+      const int j = d.hidx[h0 + h];
+      hid[h] = j;
+      dih[h] = d.dinv32[j];
+    }
+    for (int i = tid; i < nloc; i += bd) di[i] = d.dinv32[r0 + i];
+  }
+  // outer FP64 storage (global)
+  double* x = d.x + r0;
+  double* bp = d.bp + r0;
+  double* r64 = d.r + r0;
+
+  // the calling thread's own rows: g(q, i), register slot q
+  auto own_rows = [&](auto g) {
+    if constexpr (R > 0) {
+#pragma unroll
+      for (int q = 0; q < R; ++q) {
+        const int i = tid + q * bd;
+        if (i < nloc) g(q, i);
+      }
+    } else {
+      for (int i = tid; i < nloc; i += bd) g(0, i);
+    }
+  };
+
+  // this block's words start empty, its rows unmarked; the barrier of the first
+  // reduction orders that before any block polls or marks
+  if (tid < 2) st_relaxed_b128(flow_line(d, tid, lb), 0ull, 0ull);
+  for (int i = tid; i < nloc; i += bd) {
+    *flow_w32(d, 0, r0 + i) = 0ull;
+    *flow_w32(d, 1, r0 + i) = 0ull;
+    mark[r0 + i] = 0;
+  }
+  // ---- projected b and x0 ----
+  {
+    double v2[2] = {0.0, 0.0};
+    for (int i = tid; i < nloc; i += bd) {
+      v2[0] += d.b[r0 + i];
+      if (d.use_x0) v2[1] += x[i];
+    }
+    put_partials<2>(d, lb, red, v2, sh);
+    if (!grp.sync(sh)) return;
+    get_totals<2>(d, red, sh);
+    ++red;
+  }
+  for (int h = tid; h < nh; h += bd) mark[hid[h]] = 1;
+  {
+    const double mb = d.fixed ? 0.0 : sh.tot[0] / d.n, mx = d.fixed ? 0.0 : sh.tot[1] / d.n;
+    double v1[1] = {0.0};
+    for (int i = tid; i < nloc; i += bd) {
+      const double bi = is_fixed(d, r0 + i) ? 0.0 : d.b[r0 + i] - mb;
+      bp[i] = bi;
+      v1[0] += bi * bi;
+      x[i] = (d.use_x0 && !is_fixed(d, r0 + i)) ? x[i] - mx : 0.0;
+    }
+    put_partials<1>(d, lb, red, v1, sh);
+    if (!grp.sync(sh)) return;
+    get_totals<1>(d, red, sh);
+    ++red;
+  }
+  for (int i = tid; i < nloc; i += bd) pub[i] = (unsigned char)__ldcg(mark + r0 + i);
+  const double bnorm = sqrt(sh.tot[0]);
+  if (!isfinite(bnorm)) { finish(d, lb, CGP_ERR_NONFINITE, 0, 0, 0.0, 0.0, bnorm); return; }
+  if (bnorm == 0.0) {
+    for (int i = tid; i < nloc; i += bd) x[i] = 0.0;
+    finish(d, lb, CGP_OK, 0, 0, 0.0, 0.0, 0.0);
+    return;
+  }
+  // FP64 view of the local rows for the outer residual (global arrays)
+  Local L;
+  L.row = d.rowptr + r0;
+  L.col = d.col;
+  L.val = d.val;
+
+  // register rows: the first NE entries (absent ones: value 0 at the row's own
+  // position) and whether a row goes on after them
+  constexpr bool VREG = R == 1 || R == 2;            // u_(k-1) in registers too
+  float rq[NR], sq[NR], wq[NR], uq[NR], vq[NR], dq[NR], aq[NR][NE];
+  unsigned cq[NR][NE / 2];
+  unsigned out = 0, more = 0;                        // rows to publish; rows longer than NE
+  if constexpr (R > 0) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      dq[q] = rq[q] = sq[q] = wq[q] = uq[q] = vq[q] = 0.0f;
+#pragma unroll
+      for (int e = 0; e < NE; ++e) aq[q][e] = 0.0f;
+#pragma unroll
+      for (int e = 0; e < NE / 2; ++e) cq[q][e] = 0u;
+    }
+    own_rows([&](int q, int i) {
+      const int k0 = row[i], k1 = row[i + 1];
+#pragma unroll
+      for (int e = 0; e < NE; ++e) {
+        const bool in = k0 + e < k1;
+        aq[q][e] = in ? val[k0 + e] : 0.0f;
+        cq[q][e / 2] |= (unsigned)(in ? col[k0 + e] : i) << (16 * (e & 1));
+      }
+      dq[q] = di[i];
+      if (pub[i]) out |= 1u << q;
+      if (k1 - k0 > NE) more |= 1u << q;
+    });
+  }
+
+  int total = 0, sweeps = 0, status = CGP_ERR_NOT_CONVERGED;
+  double rel = 0.0;
+  while (true) {
+    // ---- FP64 residual r = bp - K x, projected; x is complete (barrier above) ----
+    {
+      double v1[1] = {0.0};
+      spmv_local<T, double>(
+          L, r0, nloc, [&](int jl) { return x[jl]; }, [&](int j) { return __ldcg(d.x + j); },
+          [&](int il, double s) {
+            const double ri = bp[il] - s;
+            r64[il] = ri;
+            v1[0] += ri;
+          });
+      put_partials<1>(d, lb, red, v1, sh);
+      if (!grp.sync(sh)) return;
+      get_totals<1>(d, red, sh);
+      ++red;
+    }
+    {
+      const double mr = d.fixed ? 0.0 : sh.tot[0] / d.n;
+      double v1[1] = {0.0};
+      for (int i = tid; i < nloc; i += bd) {
+        const double ri = r64[i] - mr;
+        v1[0] += ri * ri;
+        const float rf = (float)ri;
+        ir[i] = rf;
+        iu[i] = di[i] * rf;
+        ie[i] = 0.0f;
+        R0[r0 + i] = rf;
+      }
+      put_partials<1>(d, lb, red, v1, sh);
+      if (!grp.sync(sh)) return;   // also publishes r_0 for the ghost rows
+      get_totals<1>(d, red, sh);
+      ++red;
+    }
+    rel = sqrt(sh.tot[0]) / bnorm;
+    if (!isfinite(rel)) { status = CGP_ERR_NONFINITE; break; }
+    if (rel <= d.tol) { status = CGP_OK; break; }
+    if (sweeps >= d.max_sweeps || total >= d.max_it) { status = CGP_ERR_NOT_CONVERGED; break; }
+
+    // ---- FP32 inner solve: u_0 and the ghost rows, then iterations from the product w_0 = A u_0 ----
+    for (int i = tid; i < nloc; i += bd) ext[i] = iu[i];
+    for (int h = tid; h < nh; h += bd) {
+      const float rj = __ldcg(R0 + hid[h]);
+      gr[h] = rj;
+      ext[nloc + h] = dih[h] * rj;
+    }
+    if constexpr (R > 0) {
+      own_rows([&](int q, int i) {
+        rq[q] = ir[i];
+        uq[q] = iu[i];
+      });
+    }
+    if (tid == 0) {
+      sh.fsc[4] = (float)(d.inner_tol * d.inner_tol);
+      // below half the outer target the correction would already pass the outer test
+      const double floor = 0.5 * d.tol * bnorm;
+      sh.fsc[5] = (float)(floor * floor);
+    }
+    int k = 0;                           // products formed in this sweep, less one
+    float old[2] = {0.0f, 0.0f};         // flow_scalars_f's last gamma and alpha (warp 0)
+    bool bad = false;
+    while (true) {
+      __syncthreads();
+      // ---- w_k = A u_k, published where another block reads it; the partial sums ----
+      float v3[3] = {0.0f, 0.0f, 0.0f};
+      const unsigned tag = (unsigned)(red + 1);
+      if constexpr (R > 0) {
+        own_rows([&](int q, int i) {
+          float g[NE];
+#pragma unroll
+          for (int e = 0; e < NE; ++e) g[e] = ext[(cq[q][e / 2] >> (16 * (e & 1))) & 0xFFFFu];
+          float s = 0.0f;
+#pragma unroll
+          for (int e = 0; e < NE; ++e) s = fmaf(aq[q][e], g[e], s);
+          wq[q] = s;
+        });
+        if (more) {
+          own_rows([&](int q, int i) {
+            if (more & (1u << q))
+              for (int e = row[i] + NE; e < row[i + 1]; ++e) wq[q] = fmaf(val[e], ext[col[e]], wq[q]);
+          });
+        }
+        own_rows([&](int q, int i) {
+          if (out & (1u << q))
+            st_relaxed_u64(flow_w32(d, red, r0 + i), ((unsigned long long)tag << 32) | __float_as_uint(wq[q]));
+          v3[0] = fmaf(rq[q], uq[q], v3[0]);
+          v3[1] = fmaf(wq[q], uq[q], v3[1]);
+          v3[2] = fmaf(rq[q], rq[q], v3[2]);
+        });
+      } else {
+        flow_rows<T>(row, col, val, ext, nloc, tid, bd, [&](int il, float s) {
+          const float u = ext[il], r = ir[il];
+          iw[il] = s;
+          if (pub[il]) st_relaxed_u64(flow_w32(d, red, r0 + il), ((unsigned long long)tag << 32) | __float_as_uint(s));
+          v3[0] = fmaf(r, u, v3[0]);
+          v3[1] = fmaf(s, u, v3[1]);
+          v3[2] = fmaf(r, r, v3[2]);
+        });
+      }
+      flow_put_f(d, lb, red, act, v3, sh);
+      // ---- p_(k-1) = u_(k-1) + beta p_(k-2), e += alpha p_(k-1), while the words travel ----
+      if (k > 0) {
+        const float alpha = sh.abf[(k - 1) & 1][0], beta = sh.abf[(k - 1) & 1][1];
+        own_rows([&](int q, int i) {
+          const float uo = VREG ? vq[q] : iu[i];
+          const float pi = k == 1 ? uo : fmaf(beta, ip[i], uo);
+          ip[i] = pi;
+          ie[i] = fmaf(alpha, pi, ie[i]);
+          if (!VREG) iu[i] = R > 0 ? uq[q] : ext[i];
+        });
+      }
+      // ---- the halo's w, then the sums ----
+      if (tid >= f0) {
+        PollLimit lim(d);
+        constexpr int B = 4;   // loads of a thread in flight
+        const int nt = bd - f0;
+        for (int h = tid - f0; h < nh; h += B * nt) {
+          unsigned long long a[B];
+#pragma unroll
+          for (int q = 0; q < B; ++q)
+            a[q] = h + q * nt < nh ? ld_relaxed_u64(flow_w32(d, red, hid[h + q * nt])) : (unsigned long long)tag << 32;
+#pragma unroll
+          for (int q = 0; q < B; ++q) {
+            while ((unsigned)(a[q] >> 32) != tag && !lim.expired()) a[q] = ld_relaxed_u64(flow_w32(d, red, hid[h + q * nt]));
+            if ((unsigned)(a[q] >> 32) != tag) sh.tflag = 0;
+            if (h + q * nt < nh) gw[h + q * nt] = __uint_as_float((unsigned)a[q]);
+          }
+        }
+      }
+      if (warp < G && !flow_poll_f(d, red, warp, G, sh)) sh.tflag = 0;
+      __syncthreads();
+      if (warp == 0) flow_scalars_f(G, k, total + k >= d.max_it, old, sh);
+      __syncthreads();
+      if (!sh.tflag) return;
+      ++red;
+      const int st = sh.isc[0];
+      if (st >= 0) {
+        bad = st == 1;
+        break;
+      }
+      const float alpha = sh.abf[k & 1][0], beta = sh.abf[k & 1][1];
+      // ---- own rows and ghost rows: s, r, u_(k+1) ----
+      own_rows([&](int q, int i) {
+        const float wi = R > 0 ? wq[q] : iw[i];
+        const float si = k == 0 ? wi : fmaf(beta, R > 0 ? sq[q] : is[i], wi);
+        const float ri = fmaf(-alpha, si, R > 0 ? rq[q] : ir[i]);
+        const float ui = (R > 0 ? dq[q] : di[i]) * ri;
+        if constexpr (R > 0) {
+          sq[q] = si;
+          rq[q] = ri;
+          if (VREG) vq[q] = uq[q];
+          uq[q] = ui;
+        } else {
+          is[i] = si;
+          ir[i] = ri;
+        }
+        ext[i] = ui;
+      });
+      for (int h = bd - 1 - tid; h < nh; h += bd) {
+        const float sj = k == 0 ? gw[h] : fmaf(beta, gs[h], gw[h]);
+        gs[h] = sj;
+        const float rj = fmaf(-alpha, sj, gr[h]);
+        gr[h] = rj;
+        ext[nloc + h] = dih[h] * rj;
+      }
+      ++k;
+    }
+    total += k;
+    if (bad) { status = CGP_ERR_NONFINITE; break; }
+    // ---- FP64 correction and projection; x published for the next residual ----
+    {
+      double v1[1] = {0.0};
+      for (int i = tid; i < nloc; i += bd) {
+        const double xi = x[i] + (double)ie[i];
+        x[i] = xi;
+        v1[0] += xi;
+      }
+      put_partials<1>(d, lb, red, v1, sh);
+      if (!grp.sync(sh)) return;
+      get_totals<1>(d, red, sh);
+      ++red;
+      const double mx = d.fixed ? 0.0 : sh.tot[0] / d.n;
+      for (int i = tid; i < nloc; i += bd) x[i] -= mx;
+      if (!grp.sync(sh)) return;
+    }
+    ++sweeps;
+    if (k == 0 && total < d.max_it) { status = CGP_ERR_BREAKDOWN; break; }  // no inner progress
+  }
+  finish(d, lb, status, total, sweeps, rel, rel, bnorm);
+}
+
+// The solve loop of a system in the general kernels: dataflow iterations where
+// its rows are resident, its reductions tagged and its blocks large enough
+// (cgp_flow.cu has kernels of their own for the FP32 register rows), the barrier
+// forms otherwise.
+template <int T, bool RES>
+__device__ __forceinline__ void solve_any(const Desc& d, int lb, Shared& sh) {
+  if (d.mixed) {
+    if constexpr (RES) {
+      if (d.tagged && blockDim.x >= kFlowMinBlock) {
+        solve_mixed_flow<T, 0>(d, lb, sh);
+        return;
+      }
+    }
+    solve_mixed<T, RES>(d, lb, sh);
+  } else if (d.classic) {
+    solve_fp64<T, RES>(d, lb, sh);
+  } else {
+    if constexpr (RES) {
+      if (d.tagged && blockDim.x >= kFlowMinBlock) {
+        solve_fp64_flow<T>(d, lb, sh);
+        return;
+      }
+    }
+    solve_fp64_sr<T, RES>(d, lb, sh);
+  }
+}
+
+}  // namespace
+}  // namespace cgp

@@ -34,6 +34,8 @@ struct SolveResult {
   unsigned long long t_end;  // device clock (ns) when the solve finished
 };
 
+constexpr int kLineBytes = 128;  // one L2 line: each block's polled words sit on lines of their own
+
 // Tuning of the persistent solver launch (chosen by the autotuner or defaults).
 struct SolverTuning {
   int block;          // threads per block (0 = default)
@@ -140,12 +142,12 @@ struct cgp_mesh_impl {
   double* p2 = nullptr;
   double* q = nullptr;
   double* pub64 = nullptr;   // [18 n] published vectors: single-reduction R[2], W[2], S[2] (6 n doubles);
-                             // pipelined tagged W[3], Z[3], N[3] (9 n 16-byte words)
-  float* f32pub = nullptr;   // [6 n] mixed: published R[2], W[2], S[2]
+                             // dataflow W[2] (2 n 16-byte words) and r; pipelined tagged W[3], Z[3], N[3] (9 n words)
+  float* f32pub = nullptr;   // [6 n] mixed: published R[2], W[2], S[2]; dataflow W[2] (2 n 8-byte words) and r
   float* f32own = nullptr;   // [6 n] mixed without shared-memory residency: own inner vectors
   float* fpart = nullptr;    // [8 * max_blocks] FP32 partial sums
   double* part = nullptr;    // [max_blocks * 32] per-block fixed-point partial sums
-  unsigned long long* tpart = nullptr;  // [2][3][max_blocks] tagged 128-bit partial sums
+  unsigned long long* tpart = nullptr;  // [max_blocks][2] lines of kLineBytes: tagged partial sums by bank
   unsigned* nflag = nullptr; // [max_blocks] pipelined tiles: published-w counts of the blocks
   unsigned* bar = nullptr;   // grid barrier counter
   SolveResult* res = nullptr;

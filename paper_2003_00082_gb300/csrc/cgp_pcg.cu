@@ -35,11 +35,12 @@
 #include <string>
 #include <vector>
 
-#include "cgp_solver.cuh"
+#include "cgp_flow.cuh"
 
 namespace cgp {
 
-// kernels compiled in their own units (cgp_pcg_batch.cu, cgp_pipe.cu)
+// kernels compiled in their own units (cgp_flow.cu, cgp_pcg_batch.cu, cgp_pipe.cu)
+const void* mixed_flow_kernel_ptr(int chunk, int block, bool batched);
 const void* batched_kernel_ptr(int lanes, bool res);
 const void* pipe_kernel_ptr(int lanes, bool batched);
 
@@ -49,14 +50,10 @@ template <int T, bool RES>
 __global__ void __launch_bounds__(MAX_BLOCK) pcg_persistent_kernel(Desc d) {
   __shared__ Shared sh;
   mark_pending(d, blockIdx.x);
-  if (d.mixed)
-    solve_mixed<T, RES>(d, blockIdx.x, sh);
-  else if (d.classic)
-    solve_fp64<T, RES>(d, blockIdx.x, sh);
-  else if (RES && d.pipelined && d.stencil)
+  if (!d.mixed && RES && d.pipelined && d.stencil)
     solve_fp64_pl<T>(d, blockIdx.x, sh);
   else
-    solve_fp64_sr<T, RES>(d, blockIdx.x, sh);
+    solve_any<T, RES>(d, blockIdx.x, sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -468,6 +465,15 @@ BatchFn resident_batched_kernel_for(SolverKind& kind, int lanes, int block) {
   return batched_kernel_for(lanes, true);
 }
 
+// The mixed kernel with register rows (cgp_flow.cu) in place of `fn` where it
+// applies: tagged reductions, one lane per row, and no more rows a thread than
+// it holds.
+const void* flow_or(const void* fn, SolverKind kind, int lanes, int flags, int chunk, int block, bool batched) {
+  if (lanes != 1 || !(flags & 8) || kind != KIND_MIXED) return fn;
+  const void* f = mixed_flow_kernel_ptr(chunk, block, batched);
+  return f ? f : fn;
+}
+
 // Dynamic shared memory of a block that keeps its rows resident: the classic
 // FP64 solver needs seven vectors, the halo buffer and an FP64 CSR slice; the
 // single-reduction FP64 solver nine vectors, the halo buffer, D^-1 of the
@@ -487,6 +493,7 @@ size_t res_smem_bytes(SolverKind kind, int chunk, const HaloPlan& hp) {
     s = 8 * ((size_t)12 * chunk + 5 * (size_t)hp.max_halo + hp.max_nnz) + ints;
   else
     s = 8 * ((size_t)10 * chunk + 5 * (size_t)hp.max_halo + hp.max_nnz) + ints;
+  s += chunk;   // dataflow iterations: which rows other blocks read
   return (s + 15) / 16 * 16;
 }
 
@@ -500,11 +507,11 @@ size_t res_smem_rows(SolverKind kind, int chunk, int nnz) {
 
 // Dynamic shared memory of a resident single-reduction FP64 block on O-grid
 // tiles: nine vectors, the padded box, D^-1 of the halo, seven coefficient
-// planes, three staging buffers of the halo; box positions of the rows and
-// the halo, and the halo's global rows.
+// planes, ghost r, s, w of the halo; box positions of the rows and the halo,
+// the halo's global rows, and one byte per row.
 size_t res_smem_stencil(int chunk, int max_halo, int box_cap) {
   const size_t s = 8 * ((size_t)16 * chunk + (size_t)box_cap + 4 * (size_t)max_halo) +
-                   4 * ((size_t)chunk + 2 * (size_t)max_halo);
+                   4 * ((size_t)chunk + 2 * (size_t)max_halo) + chunk;
   return (s + 15) / 16 * 16;
 }
 
@@ -563,6 +570,8 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
   if (!m || (tu.flags & 1)) return CGP_OK;
   if (tiles) {
     const int chunk = (n + nblk - 1) / nblk;
+    // bit 4 with the tiles: the pipelined iteration, given three polling warps and five computing ones
+    const bool pl = (tu.flags & 16) && block >= 256 && nblk <= 2048;
     PcgFn fnr = pcg_kernel_for(lanes, true);
     cudaFuncAttributes fa{};
     if (cudaFuncGetAttributes(&fa, (const void*)fnr) != cudaSuccess) {
@@ -570,8 +579,6 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
       return CGP_OK;
     }
     const size_t limit = (size_t)std::max(0, optin_smem(device) - (int)fa.sharedSizeBytes - 1024);
-    // bit 4 with the tiles: the pipelined iteration, given three polling warps and five computing ones
-    const bool pl = (tu.flags & 16) && block >= 256 && nblk <= 2048;
     const size_t smem = pl ? res_smem_stencil_pl(chunk, ps->st_max_halo, ps->box_cap)
                            : res_smem_stencil(chunk, ps->st_max_halo, ps->box_cap);
     if (smem > limit) return CGP_OK;
@@ -595,6 +602,7 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
   const int rough_nnz = hrp[std::min(n, chunk)] - hrp[0];
   SolverKind kind = solver_kind(mixed, tu.flags);
   PcgFn fnr = resident_kernel_for(kind, lanes, block);
+  fnr = flow_or(fnr, kind, lanes, tu.flags, chunk, block, false);
   cudaFuncAttributes fa{};
   if (cudaFuncGetAttributes(&fa, (const void*)fnr) != cudaSuccess) {
     cudaGetLastError();
@@ -960,6 +968,9 @@ int batch_plan(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts& o) {
   bool res = !(sh.flags & 1);
   size_t smem = 0;
   BatchFn fnr = resident_batched_kernel_for(kind, lanes, block);
+  int max_chunk = 1;
+  for (int i = 0; i < count; ++i) max_chunk = std::max(max_chunk, (B->meshes[i]->n_c + nb[i] - 1) / nb[i]);
+  fnr = flow_or(fnr, kind, lanes, sh.flags, max_chunk, block, true);
   cudaFuncAttributes fa{};
   if (res && cudaFuncGetAttributes(&fa, (const void*)fnr) != cudaSuccess) {
     cudaGetLastError();
@@ -1111,6 +1122,9 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
     for (int i : grp) total += nb[i];
     bool res = can_res;
     size_t smem = 0;
+    int max_chunk = 1;
+    for (int i : grp) max_chunk = std::max(max_chunk, (B->meshes[i]->n_c + nb[i] - 1) / nb[i]);
+    const BatchFn fnw = flow_or(fnr, kind, lanes, sh.flags, max_chunk, block, true);   // this wave's kernel
     std::vector<HaloPlan> hp(count);
     for (int i : grp) {
       if (!res) break;
@@ -1128,9 +1142,9 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
     }
     if (res) {
       int per_sm = 0;
-      if (cudaFuncSetAttribute((const void*)fnr, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      if (cudaFuncSetAttribute((const void*)fnw, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)std::max(smem, max_smem)) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fnr, block, smem) != cudaSuccess) {
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fnw, block, smem) != cudaSuccess) {
         cudaGetLastError();
         per_sm = 0;
       }
@@ -1167,7 +1181,7 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
       for (int k = 0; k < nb[i]; ++k) blk_inst.push_back(i);
       blk0 += nb[i];
     }
-    waves.push_back(cgp_batch_s::Wave{total, off, res, smem, res ? fnr : fn0});
+    waves.push_back(cgp_batch_s::Wave{total, off, res, smem, res ? fnw : fn0});
   }
   if (blk_inst.size() > (size_t)sms * std::max(32, count)) return fail(CGP_ERR_INVALID_ARG, "batch: too many blocks");
   CGP_CUDA(cudaMemcpy(B->d_desc, desc.data(), sizeof(Desc) * count, cudaMemcpyHostToDevice));

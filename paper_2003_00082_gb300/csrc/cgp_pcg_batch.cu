@@ -2,7 +2,7 @@
 // cooperative launch, each on its own group of blocks (the solve loops are
 // those of the single-system kernel, cgp_solver.cuh).  Compiled as a unit of
 // its own so that it builds in parallel with the rest of the solver.
-#include "cgp_solver.cuh"
+#include "cgp_flow.cuh"
 
 namespace cgp {
 namespace {
@@ -18,12 +18,7 @@ __global__ void __launch_bounds__(MAX_BLOCK)
   const Desc& d = descs[blk_inst[blockIdx.x]];
   const int lb = blockIdx.x - d.blk0;
   mark_pending(d, lb);
-  if (d.mixed)
-    solve_mixed<T, RES>(d, lb, sh);
-  else if (d.classic)
-    solve_fp64<T, RES>(d, lb, sh);
-  else
-    solve_fp64_sr<T, RES>(d, lb, sh);
+  solve_any<T, RES>(d, lb, sh);
 }
 
 }  // namespace

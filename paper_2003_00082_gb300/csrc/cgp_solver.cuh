@@ -41,7 +41,7 @@ struct Desc {
   float* f32own;      // mixed without RES: own r, u, w, p, s, e ([6][n])
   float* fpart;       // mixed: FP32 partial slots [2][NCOMP][part_stride]
   double* part;
-  unsigned long long* tpart;  // FP64 single-reduction: tagged slots [2][3][part_stride] (128-bit)
+  unsigned long long* tpart;  // tagged slots and records: per block two lines of kLineBytes (banks by parity)
   unsigned* nflag;    // FP64 pipelined tiles: per block, the count of its published w (release)
   int part_stride;
   unsigned* bar;
@@ -88,6 +88,13 @@ __device__ __forceinline__ V warp_sum(V v) {
   return v;
 }
 
+// Barrier of nthreads threads (whole warps) on barrier id (not 0, which
+// __syncthreads uses); the warp's lanes are reconverged first.
+__device__ __forceinline__ void named_sync(int id, int nthreads) {
+  __syncwarp();
+  asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+
 struct Shared {
   unsigned long long wlo[3][32];  // per-warp fixed-point partials of one reduction
   long long whi[3][32];
@@ -100,6 +107,13 @@ struct Shared {
   float fsc[8];
   int flag;
   int tflag;                    // outcome of the last tagged reduction's wait
+  long long phi[3][8];          // dataflow iterations: the polling warps' shares of the totals
+  int pexp[3][8];
+  float pf[3][8];
+  long long bsum[3];            // ... the block's partial sums
+  int bexp[3];
+  double ab[2][2];              // ... alpha and beta by iteration parity
+  float abf[2][2];
 };
 
 // Barrier over the blocks of one instance (cgp_sync.h): a block that gives
@@ -166,9 +180,12 @@ __device__ __forceinline__ unsigned long long* part_slot(const Desc& d, int red,
 // Tagged slots (cgp_fixed.h: fx::pack_tagged): one 128-bit word per (bank,
 // component, block) that says by itself whether it holds reduction `red`, so
 // a block can read the slots while it waits for the group barrier instead of
-// after it.  A block zeroes its slots at the start of a launch.
+// after it.  A block's slots of a bank share one 128-byte line that no other
+// block writes, so pollers of different blocks do not queue on a line.  A block
+// zeroes its slots at the start of a launch.
 __device__ __forceinline__ ulonglong2* tag_slot(const Desc& d, int red, int c, int blk) {
-  return reinterpret_cast<ulonglong2*>(d.tpart) + ((size_t)((red & 1) * 3 + c) * d.part_stride + blk);
+  return reinterpret_cast<ulonglong2*>(reinterpret_cast<unsigned char*>(d.tpart) +
+                                       ((size_t)blk * 2 + (red & 1)) * kLineBytes) + c;
 }
 
 // Sum NC (<= 3) per-thread values over the block; warp c then folds
@@ -579,13 +596,13 @@ __device__ __forceinline__ int stencil_offset(int k, int Ba) {
 // y = K v over the block's own rows in the O-grid tile form: row i sits at
 // box position pos[i] and reads its seven neighbours at fixed offsets of the
 // padded box (own values, gathered halo values, zeros on the ring outside the
-// domain); no column indices.  One row per thread; op(i, s) as for spmv_ext.
+// domain); no column indices.  Rows of thread t among nt; op(i, s) as for spmv_ext.
 template <typename Op>
 __device__ __forceinline__ void spmv_box(const int* __restrict__ pos, const double* __restrict__ planes, int chunk,
-                                         const double* box, int Ba, int nloc, Op op) {
+                                         const double* box, int Ba, int nloc, int t, int nt, Op op) {
   const int o1 = stencil_offset(1, Ba), o2 = stencil_offset(2, Ba), o3 = stencil_offset(3, Ba);
   const int o4 = stencil_offset(4, Ba), o5 = stencil_offset(5, Ba), o6 = stencil_offset(6, Ba);
-  for (int i = threadIdx.x; i < nloc; i += blockDim.x) {
+  for (int i = t; i < nloc; i += nt) {
     const int q = pos[i];
     double s = planes[i] * box[q];
     s = fma(planes[chunk + i], box[q + o1], s);
@@ -997,7 +1014,7 @@ __device__ void solve_fp64_sr(const Desc& d, int lb, Shared& sh) {
   auto own_at = [&](int i) { return st ? spos[i] : i; };
   auto halo_at = [&](int h) { return st ? hpos[h] : nloc + h; };
   auto product = [&](auto op) {
-    if (st) spmv_box(spos, L.val, chunk, ext, Ba, nloc, op);
+    if (st) spmv_box(spos, L.val, chunk, ext, Ba, nloc, tid, bd, op);
     else spmv_ext<T>(L.row, L.col, L.val, ext, nloc, op);
   };
 
@@ -1322,13 +1339,6 @@ __device__ void solve_fp64_sr(const Desc& d, int lb, Shared& sh) {
 constexpr int kPlMinBlock = 256;   // three polling warps and at least five computing ones
 constexpr int kPlMaxNbr = 64;      // blocks owning a tile's halo rows (itself across the periodic seam)
 constexpr int kPlMaxBlocks = 2048; // blocks of a launch (the owners' bitmap)
-
-// Barrier of nthreads threads (whole warps) on barrier id (not 0, which
-// __syncthreads uses); the warp's lanes are reconverged first.
-__device__ __forceinline__ void named_sync(int id, int nthreads) {
-  __syncwarp();
-  asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
 
 template <int T>
 __device__ void solve_fp64_pl(const Desc& d, int lb, Shared& sh) {
@@ -1688,7 +1698,8 @@ __device__ void solve_fp64_pl(const Desc& d, int lb, Shared& sh) {
 // red + 1 high, in the tagged-slot area (a single-copy atomic store; the
 // block zeroes its words at launch start).  Banks by the reduction's parity.
 __device__ __forceinline__ unsigned long long* ftag_slot(const Desc& d, int red, int c, int blk) {
-  return reinterpret_cast<unsigned long long*>(d.tpart) + ((size_t)((red & 1) * 3 + c) * d.part_stride + blk);
+  return reinterpret_cast<unsigned long long*>(reinterpret_cast<unsigned char*>(d.tpart) +
+                                               ((size_t)blk * 2 + (red & 1)) * kLineBytes) + c;
 }
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
