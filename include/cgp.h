@@ -280,7 +280,8 @@ int cgp_poisson_solve_noalloc(int n, const int* rowptr, const int* col, const do
  *                     bit 4: pipelined FP64 iteration, as for
  *                     cgp_set_tuning; bits 5-6: waves
  *                     with 256 << k rows per block).  INVALID_ARG for other
- *                     bits.
+ *                     bits.  All zero (as after cgp_batch_create): waves with
+ *                     tagged reductions where rows fit in shared memory.
  * cgp_batch_autotune  times a set of launch shapes on the batch's own
  *                     systems (from x = 0) and keeps the fastest; writes the
  *                     best time in ms to best_ms (nullable).  Synchronous;
@@ -472,6 +473,11 @@ int cgp_mesh_set_ogrid(cgp_mesh m, int n_theta, int n_r);
  *         try this form); other bits must be 0.
  *         SpMV: bit 0 uses the O-grid stencil form (cgp_mesh_set_ogrid) with
  *         one thread per row (lanes ignored).
+ * All zero (as after cgp_assemble) lets the solver choose: tagged reductions
+ * with rows in shared memory where they fit; FP64 about 96 rows per block, on
+ * O-grid tiles (registered meshes) or, from 4096 rows on, in the bisection
+ * order (the renumbered system is built by the first solve); MIXED about 256
+ * rows per block.
  * Invalid shapes are rejected with INVALID_ARG.  cgp_autotune sets these.
  */
 typedef enum {

@@ -634,6 +634,35 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
   return CGP_OK;
 }
 
+// Launch of a mesh that was never tuned (tuning all zero; `tu` receives the
+// shape used).  The dataflow iterations (flag bit 3) wherever rows fit in shared
+// memory, 512 threads a block.  FP64: about 96 rows a block, since the exchange
+// costs nearly the same for any number of blocks while the FP64 pipe of every SM
+// takes its share of the rows (128x64: 1.32 ms on 76 blocks, 1.99 ms on 35 with
+// 256 rows; 64x32: 0.60 ms on 24, 0.91 ms on 9); O-grid tiles where the mesh is
+// registered (512x256: 8.3 ms against 9.0 ms in the bisection order and 11.0 ms
+// in the mesh's own), else the bisection order from 4096 rows on (321x163: 4.0
+// against 4.4 ms), below which it gains nothing.  MIXED: 256 rows a block in the
+// mesh's order (64x32 0.43 ms with 9 blocks, 0.44 with 24; bisection gains under
+// 1 % at any size and costs a second copy of the system).  Systems whose rows do
+// not fit keep the barrier forms with rows in global memory.
+int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps, SolverTuning& tu) {
+  const int n = m->n_c, sms = std::max(1, dev_info(m->device).sms);
+  const int rows = mixed ? 256 : 96;
+  const int nblk = std::min(sms, std::max(1, (n + rows - 1) / rows));
+  int flags[3], count = 0;
+  if (!mixed && nblk > 1 && m->st_nt > 0) flags[count++] = 40;
+  if (!mixed && n >= 4096) flags[count++] = 12;
+  flags[count++] = 8;
+  for (int k = 0; k < count; ++k) {
+    tu = SolverTuning{512, 1, nblk, flags[k]};
+    // a renumbered system that cannot be allocated is no reason to refuse the solve
+    if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.res) return CGP_OK;
+  }
+  tu = SolverTuning{0, 0, 0, 0};
+  return plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps);
+}
+
 }  // namespace
 
 int solver_max_blocks(int device) {
@@ -718,10 +747,12 @@ __global__ void perm_scatter_kernel(int n, const int* __restrict__ perm, const d
 int launch_solve(cgp_mesh_impl* m, const double* b, double* x, const cgp_solve_opts& o, cgp_solve_info* info_dev,
                  cudaStream_t s) {
   const bool mixed = o.precision == CGP_MIXED;
-  const SolverTuning& tu = m->tune[mixed ? CGP_TUNE_SOLVE_MIXED : CGP_TUNE_SOLVE_FP64];
+  SolverTuning tu = m->tune[mixed ? CGP_TUNE_SOLVE_MIXED : CGP_TUNE_SOLVE_FP64];
   LaunchPlan plan;
   PermSystem* ps = nullptr;
-  int st = plan_solve(m, m->device, m->n_c, m->max_blocks, tu, mixed, plan, &ps);
+  int st = tu.block == 0 && tu.lanes == 0 && tu.blocks == 0 && tu.flags == 0
+               ? plan_default(m, mixed, plan, &ps, tu)
+               : plan_solve(m, m->device, m->n_c, m->max_blocks, tu, mixed, plan, &ps);
   if (st != CGP_OK) return st;
   const int nblk = plan.nblk;
   // barrier epochs stay far below 2^32 / nblk
@@ -1053,6 +1084,9 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
   const int lanes = sh.lanes > 0 ? sh.lanes : 1;
   const int block = sh.block > 0 ? sh.block : 512;
   const bool mixed = o.precision == CGP_MIXED;
+  // never tuned: tagged reductions (dataflow iterations) where a wave's rows are resident
+  const bool untuned = sh.block == 0 && sh.lanes == 0 && sh.per_sm == 0 && sh.flags == 0;
+  const int flags = untuned ? 8 : sh.flags;
   BatchFn fn0 = batched_kernel_for(lanes, false);
   if (!fn0 || block < 64 || block > MAX_BLOCK || block % 32 != 0 || block % lanes != 0)
     return fail(CGP_ERR_INVALID_ARG, "batch tuning: bad block or lanes");
@@ -1124,7 +1158,7 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
     size_t smem = 0;
     int max_chunk = 1;
     for (int i : grp) max_chunk = std::max(max_chunk, (B->meshes[i]->n_c + nb[i] - 1) / nb[i]);
-    const BatchFn fnw = flow_or(fnr, kind, lanes, sh.flags, max_chunk, block, true);   // this wave's kernel
+    const BatchFn fnw = flow_or(fnr, kind, lanes, flags, max_chunk, block, true);   // this wave's kernel
     std::vector<HaloPlan> hp(count);
     for (int i : grp) {
       if (!res) break;
@@ -1175,7 +1209,7 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
       }
       unsigned char* ctrl = B->d_ctrl + kCtrlPerInstance * i;
       desc[i] = make_desc(m, B->b[i], B->x[i], o, nb[i], lp, reinterpret_cast<unsigned*>(ctrl),
-                          reinterpret_cast<SolveResult*>(ctrl + 256), sh.flags);
+                          reinterpret_cast<SolveResult*>(ctrl + 256), untuned && !res ? 0 : flags);
       desc[i].blk0 = blk0;
       if (max_epochs(o) * nb[i] >= (1LL << 31)) return fail(CGP_ERR_INVALID_ARG, "batch: max_it too large");
       for (int k = 0; k < nb[i]; ++k) blk_inst.push_back(i);
