@@ -396,8 +396,9 @@ int cgp_lorentz(cgp_mesh m, const double* phi_f, const double* u_f, const double
  * gradients of the fine triangles around the node.
  * p_f, u_t, v_t, u, v  device [n_f]; u, v may alias u_t, v_t.
  * dt_over_rho          dt / rho.
- * The first call on a mesh builds the fine node -> triangle incidence
- * (synchronous, one allocation of about 24 t_f bytes, freed with the mesh).
+ * The first call on a mesh builds the correction's operator, a row of weights
+ * per fine node (synchronous; one allocation of about 72 t_f bytes, freed with
+ * the mesh, and about 26 t_f bytes while it is built).
  */
 int cgp_velocity_correct(cgp_mesh m, const double* p_f, const double* u_t, const double* v_t,
                          double dt_over_rho, double* u, double* v, void* stream);

@@ -129,6 +129,7 @@ struct cgp_mesh_impl {
   int* edges = nullptr;      // [2 * all levels' edges]: level 0 (the coarse edges, n_e of them) first
   int* tri_par = nullptr;    // [3 t_par] parents of the fine triangles (tri_c when levels == 1)
   int* mid_par = nullptr;    // [3 t_par] their midpoints m_ab, m_bc, m_ca (tri_mid when levels == 1)
+  double* shape_par = nullptr;  // [t_par][4] (b_1, b_2, c_1, c_2) 2 / a2 of the fine triangles' parents
   double* xy_f = nullptr;    // [n_f * 2] interleaved
   double* xy_c = nullptr;    // [n_c * 2]
   int* inc_ptr = nullptr;    // [n_c + 1] node -> incident triangles
@@ -170,11 +171,12 @@ struct cgp_mesh_impl {
   float* dinvd32 = nullptr;
   void* dir_base = nullptr;
 
-  // fine node -> incident fine triangles, each entry the other two vertices in
-  // counter-clockwise order (built on the first velocity correction)
-  int* vinc_ptr = nullptr;   // [n_f + 1]
-  int* vinc = nullptr;       // [3 t_f][2]
-  void* vinc_base = nullptr;
+  // operator of the velocity correction (built on the first one), rows in slices of 32:
+  // entry e of row i at vop_off[i / 32] + 32 e + i % 32
+  long long* vop_off = nullptr;   // [ceil(n_f / 32) + 1]
+  int* vop_col = nullptr;         // [vop_off's last]
+  double* vop_coef = nullptr;     // [vop_off's last][2] weights of the mean gradient's x and y
+  void* vop_base = nullptr;
 
   std::vector<HaloPlan> plans;   // cached per block count
   std::vector<PermSystem> psys;  // cached per (block count, boundary condition, tiles)
@@ -188,6 +190,7 @@ int launch_restrict_rhs(cgp_mesh_impl* m, int kind, double bz, double rho_over_d
                         const double* u_f, const double* v_f, double* u_c, double* v_c,
                         double* b, cudaStream_t s);
 int launch_prolong(cgp_mesh_impl* m, const double* xc, double* xf, cudaStream_t s);
+int launch_parent_shape(cgp_mesh_impl* m, cudaStream_t s);
 int launch_velocity_correct(cgp_mesh_impl* m, const double* p_f, const double* u_t, const double* v_t,
                             double dt_over_rho, double* u, double* v, cudaStream_t s);
 int launch_lorentz(cgp_mesh_impl* m, const double* phi, const double* u, const double* v,

@@ -290,7 +290,7 @@ extern "C" int cgp_assemble(const double* xy_c, int n_c, const int* tri_c, int t
          o_Gy = take(nz * 8), o_dinv = take(n * 8), o_K32 = take(nz * 4), o_d32i = take(n * 4),
          o_tri = take(3 * (size_t)t_c * 4), o_mid = take(3 * (size_t)t_c * 4),
          o_edges = take(2 * (size_t)m->h_lvl_eoff[levels] * 4), o_tpar = take(m->h_tri_par.size() * 4),
-         o_mpar = take(m->h_mid_par.size() * 4), o_xyf = take(2 * (size_t)m->n_f * 8),
+         o_mpar = take(m->h_mid_par.size() * 4), o_xyf = take(2 * (size_t)m->n_f * 8), o_shape = take(4 * (size_t)m->t_par * 8),
          o_xyc = take(2 * n * 8), o_incp = take((n + 1) * 4), o_inc = take(3 * (size_t)t_c * 4),
          o_bp = take(n * 8), o_r = take(n * 8), o_z = take(n * 8), o_p = take(n * 8), o_p2 = take(n * 8), o_q = take(n * 8),
          o_pub64 = take(18 * n * 8), o_f32pub = take(6 * n * 4), o_f32own = take(6 * n * 4),
@@ -317,6 +317,7 @@ extern "C" int cgp_assemble(const double* xy_c, int n_c, const int* tri_c, int t
   m->mid_par = levels >= 2 ? (int*)(base + o_mpar) : m->tri_mid;
   m->xy_f = (double*)(base + o_xyf);
   m->xy_c = (double*)(base + o_xyc);
+  m->shape_par = (double*)(base + o_shape);
   m->inc_ptr = (int*)(base + o_incp);
   m->inc_tri = (int*)(base + o_inc);
   m->bp = (double*)(base + o_bp);
@@ -353,7 +354,7 @@ extern "C" int cgp_assemble(const double* xy_c, int n_c, const int* tri_c, int t
       (st = up(m->xy_c, xy_c, 2 * n * 8)) || (st = up(m->inc_ptr, inc_ptr.data(), (n + 1) * 4)) ||
       (st = up(m->inc_tri, inc.data(), 3 * (size_t)t_c * 4)))
     return cleanup_fail(st);
-  if ((st = launch_assemble_values(m, 0))) return cleanup_fail(st);
+  if ((st = launch_assemble_values(m, 0)) || (st = launch_parent_shape(m, 0))) return cleanup_fail(st);
   e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cleanup_fail(cuda_fail(e, "assemble kernels"));
   *out = m;
@@ -518,7 +519,7 @@ extern "C" int cgp_mesh_destroy(cgp_mesh m) {
   cudaDeviceSynchronize();
   for (auto& pl : m->plans)
     if (pl.base) cudaFree(pl.base);
-  if (m->vinc_base) cudaFree(m->vinc_base);
+  if (m->vop_base) cudaFree(m->vop_base);
   if (m->dir_base) cudaFree(m->dir_base);
   for (auto& ps : m->psys) {
     if (ps.base) cudaFree(ps.base);
