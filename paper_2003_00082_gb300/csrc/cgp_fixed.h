@@ -176,39 +176,5 @@ CGP_HD inline I128 tagged_mantissa(uint64_t lo, uint64_t hi) {
   return ((I128)mh << 56) | (I128)(lo >> 8);
 }
 
-// Record: one block's three 64-bit partials S[c] (|S[c]| < 2^62, value
-// S[c] 2^(E[c] - 1074), E[c] = kBadExp for a non-finite one) of reduction
-// `red` in four 64-bit words, each with an 8-bit tag of its own, so that a
-// reader that sees the tag in all four holds one reduction's words whatever
-// the order in which they became visible:
-//   w[c] = S[c][0:56) << 8 | tag,   w[3] = (S[c] >> 56, 7 bits each; E[c],
-//   11 bits each) << 8 | tag.
-// The reductions that a record's words can hold while it is polled lie less
-// than 255 apart, and the tag is never 0 (a cleared record).
-CGP_HD inline uint64_t record_tag(int red) { return 1u + (unsigned)red % 255u; }
-CGP_HD inline void pack_record(const int64_t (&S)[3], const int (&E)[3], int red, uint64_t (&w)[4]) {
-  const uint64_t tag = record_tag(red);
-  uint64_t top = 0;
-  for (int c = 0; c < 3; ++c) {
-    const bool bad = E[c] >= 0x7FF;
-    const int64_t s = bad ? 0 : S[c];
-    w[c] = ((uint64_t)s << 8) | tag;
-    top |= ((uint64_t)(s >> 56) & 0x7Full) << (7 * c);
-    top |= (uint64_t)(bad ? 0x7FF : E[c]) << (21 + 11 * c);
-  }
-  w[3] = (top << 8) | tag;
-}
-CGP_HD inline bool record_current(const uint64_t (&w)[4], uint64_t tag) {
-  return (((w[0] ^ tag) | (w[1] ^ tag) | (w[2] ^ tag) | (w[3] ^ tag)) & 0xFFull) == 0;
-}
-CGP_HD inline int record_exponent(const uint64_t (&w)[4], int c) {
-  const int e = (int)((w[3] >> (29 + 11 * c)) & 0x7FFull);
-  return e == 0x7FF ? kBadExp : e;
-}
-CGP_HD inline int64_t record_mantissa(const uint64_t (&w)[4], int c) {
-  const int64_t hi = (int64_t)((w[3] >> (8 + 7 * c)) << 57) >> 1;   // sign and bits 56 .. 62
-  return hi | (int64_t)(w[c] >> 8);
-}
-
 }  // namespace fx
 }  // namespace cgp

@@ -3,33 +3,39 @@
 //
 // A block needs two things from the others every iteration: the totals of the
 // three dot products, and w = K u of the rows its product reads (its halo).
-// Both travel in words that show by themselves whether they are the ones
-// waited for, so a reader polls exactly the data it will use:
-//   - every block owns one 128-byte line per bank (two banks by parity) and
-//     stores its partial sums there as one record: FP64 four 64-bit words, each
-//     tagged (fx::pack_record), FP32 one tagged 128-bit word;
-//   - w of a row that another block reads is stored with the reduction's
-//     number in one 128-bit (FP64) or 64-bit (FP32) word.
+// They travel in words that show by themselves whether they are the ones waited
+// for, so a reader polls exactly the data it will use:
+//   - partial sums in tagged 128-bit words (FP64: one per component, {sum,
+//     exponent and reduction number}; FP32: one for all three) on lines that no
+//     other block writes;
+//   - w of a row that another block reads, with the reduction's number, in one
+//     128-bit (FP64) or 64-bit (FP32) word.
 // The halo rows' r and s are not published at all: a reader keeps copies of
 // them (ghost rows) and applies the owner's own operations to them every
 // iteration, so both hold the same bits.
 //
-// A bank is rewritten two reductions later.  A block stores its sums of
-// reduction k + 1 only after it has read all it needs of reduction k (the
-// stored sums depend on what it read), and reduction k + 2's words only after
-// it has seen every block's sums of k + 1, so no word is overwritten before
-// its readers have it.
+// The FP64 sums travel in two parts.  (r,u) and (r,r) are known as soon as r is
+// updated, before the product: they go out first (the early words), and their
+// exchange, decoding, the stop test and beta cost nothing, because the product
+// runs meanwhile on other warps.  Only (w,u) is left after the product (the late
+// word): one component to sum, store, poll and convert, and one quotient.
+// Meanwhile the warps with rows form p, x and s = w + beta s.
+//
+// Words of a kind live in two banks by the parity of the reduction.  A block
+// stores its early words of k + 1 after it has read every late word of k, and
+// its late word of k + 1 after it has read all early and late words of k (the
+// stored sums depend on what it read); it overwrites a bank at k + 2 only after
+// it has seen every block's words of k + 1, so no word is overwritten before its
+// readers have it.
 //
 // What bounds it: 152 blocks that exchange one flag each way take 8.1k clocks
 // an exchange through a release/acquire counter, 5.4k through slots 16 bytes
 // apart (the pollers queue on the shared lines), 3.5k through slots on lines
 // of their own stored with release, 2.6k stored relaxed; a line read on the
-// other die just after it was written costs about 1.7k of that.  Polling
-// loads the same network that the words travel on: one 32-byte load per block
-// and round is faster than three 16-byte ones (2.6k against 3.7k clocks from the
-// block barrier to the last share at 512x256).  The rest of
-// an iteration is a chain of short steps (warp sums, block sums, totals,
-// scalars), each of which is written for latency here.
+// other die just after it was written costs about 1.7k of that.  Polling loads
+// the same network that the words travel on, so a round has one lane and one
+// load per block.  The rest of an iteration is a chain of short steps (warp
+// sums, block sums, totals, scalars), each written for latency here.
 #pragma once
 
 #include "cgp_solver.cuh"
@@ -39,9 +45,9 @@ namespace {
 
 constexpr int kMaxShares = 8;   // groups of blocks whose records are folded by one warp each
 
-// This block's line of bank (red & 1).
-__device__ __forceinline__ unsigned char* flow_line(const Desc& d, int red, int blk) {
-  return reinterpret_cast<unsigned char*>(d.tpart) + ((size_t)blk * 2 + (red & 1)) * kLineBytes;
+// A block's line of bank (red & 1): kind 0 early words, 1 the late word.
+__device__ __forceinline__ unsigned char* flow_line(const Desc& d, int kind, int red, int blk) {
+  return reinterpret_cast<unsigned char*>(d.tpart) + ((size_t)blk * 4 + 2 * kind + (red & 1)) * kLineBytes;
 }
 
 // Limit of a polling loop: d.spin_ns of wall-clock time, or as soon as another
@@ -66,12 +72,42 @@ struct PollLimit {
   }
 };
 
+// One-shot signals inside a block on shared-memory barriers of one arrival a
+// phase: the waiting warps are suspended by the hardware, so they neither take
+// issue slots from the warps at work (spinning on a shared word made small
+// systems 10 % slower) nor poll the network before there can be anything to
+// read.  `phase` is the parity of the signals given before.
+__device__ __forceinline__ unsigned shared_address(const void* p) {
+  return (unsigned)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void signal_init(unsigned long long* mb) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(shared_address(mb)) : "memory");
+}
+__device__ __forceinline__ void signal_give(unsigned long long* mb) {
+  asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(shared_address(mb)) : "memory");
+}
+__device__ __forceinline__ bool signal_wait(unsigned long long* mb, unsigned phase, const Desc& d) {
+  PollLimit lim(d);
+  while (true) {
+    unsigned done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(shared_address(mb)), "r"(phase)
+        : "memory");
+    if (done) return true;
+    if (lim.expired()) return false;
+  }
+}
+
 // Groups the blocks of a solve are polled in (32 blocks a pass each) by at most
 // `most` warps.
 __device__ __forceinline__ int flow_groups(int nblk, int most) {
-  return min(min((nblk + 31) / 32, most), kMaxShares);
+  const int g = (nblk + 31) / 32, m = most < kMaxShares ? most : kMaxShares;
+  return g < m ? g : m;
 }
-
 // Row il's product with columns and values in shared memory (columns renumbered
 // into ext), its entries taken eight at a time with their loads issued together
 // (a row of a triangular mesh has about seven).
@@ -120,92 +156,81 @@ __device__ __forceinline__ void flow_rows(const int* __restrict__ row, const int
 
 // ---- FP64 -------------------------------------------------------------------
 
-__device__ __forceinline__ void st_relaxed_v4(void* p, const uint64_t (&w)[4]) {
-  asm volatile("st.relaxed.gpu.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(w[0]), "l"(w[1]), "l"(w[2]),
-               "l"(w[3])
-               : "memory");
-}
-__device__ __forceinline__ void ld_relaxed_v4(const void* p, uint64_t (&w)[4]) {
-  asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];"
-               : "=l"(w[0]), "=l"(w[1]), "=l"(w[2]), "=l"(w[3])
-               : "l"(p)
-               : "memory");
+// Word of a component: {sum S, exponent E << 48 | reduction + 1}, value
+// S 2^(E - 1074), |S| < 2^62.
+__device__ __forceinline__ void st_sum(void* p, int red, long long S, int E) {
+  st_relaxed_b128(p, (unsigned long long)S, ((unsigned long long)E << 48) | (unsigned)(red + 1));
 }
 
-// The block's partial sums of three per-thread values, stored as its record of
-// reduction `red`.  Images as in put_partials64: exact up to the truncation of
-// each term 2^-54 below the largest one of its warp or block.  Only the first
-// `act` warps have rows; after the block barrier inside, warps fw .. fw + 2 fold
-// a component each and warp fw stores the record.
-__device__ __forceinline__ void flow_put(const Desc& d, int lb, int red, int act, int fw, const double (&v)[3],
-                                         Shared& sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (warp < act) {
-    int E[3];
-    long long S[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) E[c] = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx64_exponent(v[c]));
-#pragma unroll
-    for (int c = 0; c < 3; ++c) S[c] = warp_sum57(E[c] < fx::kBadExp ? fx64_image(v[c], E[c]) : 0ll);
-    if (lane < 3) {
-      sh.whi[lane][warp] = lane == 0 ? S[0] : (lane == 1 ? S[1] : S[2]);
-      sh.wexp[lane][warp] = lane == 0 ? E[0] : (lane == 1 ? E[1] : E[2]);
-    }
-  }
-  if (threadIdx.x == 0) sh.tflag = 1;
-  __syncthreads();
-  const int c = warp - fw;
-  if (c >= 0 && c < 3) {
-    const long long sw = lane < act ? sh.whi[c][lane] : 0ll;
-    const int ew = lane < act ? sh.wexp[c][lane] : 1;
-    const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)ew);
-    const long long S = warp_sum57(E < fx::kBadExp ? (sw >> min(E - ew + 5, 63)) : 0ll);
-    if (lane == 0) {
-      sh.bsum[c] = S;
-      sh.bexp[c] = E;
-    }
-    named_sync(2, 96);
-    if (c == 0 && lane == 0) {
-      const int64_t Sa[3] = {S, sh.bsum[1], sh.bsum[2]};
-      const int Ea[3] = {E, sh.bexp[1], sh.bexp[2]};
-      uint64_t w[4];
-      fx::pack_record(Sa, Ea, red, w);
-      st_relaxed_v4(flow_line(d, red, lb), w);
-    }
+// Exact warp sum of one value per lane, as put_partials64 forms it (each term
+// truncated 2^-54 below the warp's largest), into the block's table.
+__device__ __forceinline__ void flow_warp_sum(double v, int c, int slot, Shared& sh) {
+  const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx64_exponent(v));
+  const long long S = warp_sum57(E < fx::kBadExp ? fx64_image(v, E) : 0ll);
+  if ((threadIdx.x & 31) == 0) {
+    sh.whi[c][slot] = S;
+    sh.wexp[c][slot] = E;
   }
 }
+// One warp: the block's sum of component c over `act` warps, stored at p.
+__device__ __forceinline__ void flow_block_sum(int c, int act, void* p, int red, Shared& sh) {
+  const int lane = threadIdx.x & 31;
+  const long long sw = lane < act ? sh.whi[c][lane] : 0ll;
+  const int ew = lane < act ? sh.wexp[c][lane] : 1;
+  const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)ew);
+  const long long S = warp_sum57(E < fx::kBadExp ? (sw >> min(E - ew + 5, 63)) : 0ll);
+  if (lane == 0) st_sum(p, red, S, E);
+}
 
-// Polling warp q < G: wait for the records of the blocks 32 q + lane (+ 32 G
-// ...) of reduction `red`; the warp's share of the totals goes to
-// sh.phi/pexp[c][q], value phi 2^(pexp - 1074), |phi| < 2^62.  A block's
-// partial enters with 57 bits relative to the largest one.  False (on every
-// lane) when the wait gave up.
-__device__ __forceinline__ bool flow_poll(const Desc& d, int red, int q, int G, Shared& sh) {
+// Polling warp q < G: wait for NC words of kind `kind` of the blocks 32 q + lane
+// (+ 32 G ...); the warp's shares of the totals go to sh.phi/pexp[c0 + c][q],
+// value phi 2^(pexp - 1074), |phi| < 2^62.  A block's partial enters with 57
+// bits relative to the largest one.  The warp that has the early words (kind 0)
+// loads its late word at once, into `late`, so that the load travels while the
+// early words are decoded; the wait for the late words (kind 1) starts from
+// `late`.  False (on every lane) when the wait gave up.
+template <int NC>
+__device__ __forceinline__ bool flow_poll(const Desc& d, int kind, int red, int q, int G, int c0, ulonglong2& late,
+                                          Shared& sh) {
   const int lane = threadIdx.x & 31;
   PollLimit lim(d);
-  const uint64_t tag = fx::record_tag(red);
-  long long acc[3] = {0, 0, 0};
-  int Ea[3] = {1, 1, 1};
+  const unsigned tag = (unsigned)(red + 1);
+  long long acc[NC];
+  int Ea[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    acc[c] = 0;
+    Ea[c] = 1;
+  }
   for (int base = 32 * q; base < d.nblk; base += 32 * G) {
     const int j = base + lane;
-    uint64_t w[4];
-    const void* line = flow_line(d, red, j < d.nblk ? j : base);
+    const unsigned char* line = flow_line(d, kind, red, j < d.nblk ? j : base);
+    ulonglong2 w[NC];
+    bool loaded = kind == 1 && base == 32 * q;
+    if (loaded) w[0] = late;
     while (true) {
-      ld_relaxed_v4(line, w);
-      if (__all_sync(0xffffffffu, fx::record_current(w, tag))) break;
+      bool have = true;
+      if (!loaded) {
+#pragma unroll
+        for (int c = 0; c < NC; ++c) w[c] = ld_relaxed_b128(line + 16 * c);
+      }
+      loaded = false;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) have = have && (unsigned)w[c].y == tag;
+      if (__all_sync(0xffffffffu, have)) break;
       if (__any_sync(0xffffffffu, lim.expired())) return false;
     }
-    int E[3];
-    long long S[3];
+    if (kind == 0 && base + 32 * G >= d.nblk) late = ld_relaxed_b128(flow_line(d, 1, red, min(32 * q + lane, d.nblk - 1)));
+    int E[NC];
+    long long S[NC];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int e = j < d.nblk ? fx::record_exponent(w, c) : 1;
-      S[c] = j < d.nblk ? (long long)fx::record_mantissa(w, c) : 0ll;
+    for (int c = 0; c < NC; ++c) {
+      const int e = j < d.nblk ? (int)(w[c].y >> 48) : 1;
       E[c] = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-      S[c] = E[c] < fx::kBadExp ? (S[c] >> min(E[c] - e + 5, 63)) : 0ll;
+      S[c] = j < d.nblk && E[c] < fx::kBadExp ? ((long long)w[c].x >> min(E[c] - e + 5, 63)) : 0ll;
     }
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < NC; ++c) {
       const long long t = warp_sum57(S[c]);
       if (base == 32 * q) {
         acc[c] = t;
@@ -217,9 +242,9 @@ __device__ __forceinline__ bool flow_poll(const Desc& d, int red, int q, int G, 
       }
     }
   }
-  if (lane < 3) {
-    sh.phi[lane][q] = lane == 0 ? acc[0] : (lane == 1 ? acc[1] : acc[2]);
-    sh.pexp[lane][q] = lane == 0 ? Ea[0] : (lane == 1 ? Ea[1] : Ea[2]);
+  if (lane < NC) {
+    sh.phi[c0 + lane][q] = NC == 2 && lane == 1 ? acc[NC - 1] : acc[0];
+    sh.pexp[c0 + lane][q] = NC == 2 && lane == 1 ? Ea[NC - 1] : Ea[0];
   }
   return true;
 }
@@ -231,6 +256,16 @@ __device__ __forceinline__ double scaled_double(long long X, int E) {
   const int e = (int)((fx::dbits(y) >> 52) & 0x7FF) + E - 1074;
   if (X != 0 && e > 0 && e < 0x7FF) return fx::from_bits(fx::dbits(y) + ((uint64_t)(int64_t)(E - 1074) << 52));
   return fx::to_double((fx::I128)X, E >= fx::kBadExp ? E : E + kSlot64Shift);   // NaN for a non-finite term
+}
+
+// One warp: the total of component c from its G shares, on every lane.
+__device__ __forceinline__ double flow_total(int c, int G, const Shared& sh) {
+  const int lane = threadIdx.x & 31;
+  const long long x = lane < G ? sh.phi[c][lane] : 0ll;
+  const int e = lane < G ? sh.pexp[c][lane] : 1;
+  const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+  const long long X = warp_sum57(E < fx::kBadExp ? (x >> min(E - e + 3, 63)) : 0ll);   // eight shares of 59 bits
+  return scaled_double(X, E + 3);
 }
 
 // A reciprocal of a normal a to about 22 bits, its exponent set by integer
@@ -249,80 +284,60 @@ __device__ __forceinline__ bool moderate(double a) {   // a positive normal with
   return e > 64 && e < 1982;
 }
 
-// One warp: the totals of the shares and the scalars of the next update.  An
-// FP64 operation takes 64 clocks from issue to use whatever the number of
+// The scalars of an iteration, by one warp:
+//   beta = gamma / gamma_old, alpha = gamma / (delta - beta gamma / alpha_old).
+// An FP64 operation takes 64 clocks from issue to use whatever the number of
 // active lanes, and the compiler's division about nine of them in a chain (564
-// clocks), so the lanes share the work: lane 0 forms the quotient alpha by one
-// residual correction (Markstein's) with the reciprocal that lane 1 refines
-// meanwhile by one Newton step, while lane 2 refines 1 / gamma for the next
-// iteration: three operations after the denominator.
-//   beta = gamma / gamma_old, alpha = gamma / (delta - beta gamma / alpha_old);
-// ab[k & 1] alpha and beta (two copies: the update of p and x still reads the
-// last ones), sc[4] the stop bound, sc[5] (r,r), isc[0] the stop status.
-// Keeps inv[0] = 1 / gamma_old and inv[1] = 1 / (gamma_old alpha_old); returns
-// what flow_scalars_rest needs to form the next ones off the critical path.
-struct ScalarRest {
-  double t, e, den;
+// clocks).  What depends on gamma and (r,r) alone is done while the product runs
+// (flow_early); after delta one operation gives the denominator, and the
+// quotient takes three more: lane 0 forms it by one residual correction
+// (Markstein's) with the reciprocal that lane 1 refines meanwhile by one Newton
+// step (flow_late).
+struct EarlyScalars {
+  double g, rr, m;         // gamma, (r,r), -gamma^2
+  double inv_g, inv_ga;    // 1 / gamma and, of the iteration before, 1 / (gamma alpha)
+  double den;              // denominator of alpha
+  int st;                  // stop status so far (-1: go on)
 };
-__device__ __forceinline__ ScalarRest flow_scalars(int G, int k, bool last, const double (&inv)[2], Shared& sh) {
+// Leaves beta in sh.eb[k & 1] and gives sig[0] once it is there.
+__device__ __forceinline__ void flow_early(EarlyScalars& q, int G, int k, bool last, Shared& sh) {
+  q.g = flow_total(0, G, sh);
+  const double beta = k > 0 ? q.g * q.inv_g : 0.0;
+  if ((threadIdx.x & 31) == 0) {
+    sh.eb[k & 1] = beta;
+    signal_give(&sh.sig[0]);
+  }
+  q.rr = flow_total(1, G, sh);
+  q.st = -1;
+  if (!finite_bits(q.g) || !finite_bits(q.rr)) q.st = CGP_ERR_NONFINITE;
+  else if (nonneg_le(q.rr, sh.sc[4])) q.st = CGP_OK;   // (r,r) and (tol |b|)^2 are >= 0
+  else if (last) q.st = CGP_ERR_NOT_CONVERGED;
+  q.m = -q.g * q.g;
+  q.inv_g = 1.0 / q.g;
+  if ((threadIdx.x & 31) == 0) sh.sc[5] = q.rr;
+}
+// Leaves alpha in sh.ea[k & 1] and the stop status in sh.isc[0].
+__device__ __forceinline__ void flow_late(EarlyScalars& q, int G, int k, Shared& sh) {
   const int lane = threadIdx.x & 31;
-  int E[3];
-  long long X[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    X[c] = lane < G ? sh.phi[c][lane] : 0ll;
-    const int e = lane < G ? sh.pexp[c][lane] : 1;
-    E[c] = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-    X[c] = E[c] < fx::kBadExp ? (X[c] >> min(E[c] - e + 3, 63)) : 0ll;   // eight shares of 59 bits
-  }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) X[c] = warp_sum57(X[c]);
-  const double v = scaled_double(lane == 1 ? X[1] : (lane == 2 ? X[2] : X[0]),
-                                 (lane == 1 ? E[1] : (lane == 2 ? E[2] : E[0])) + 3);
-  const double g = __shfl_sync(0xffffffffu, v, 0), dl = __shfl_sync(0xffffffffu, v, 1);
-  double beta = 0.0, den = dl;
-  if (k > 0) {
-    const double m = (lane == 0 ? -g : g) * (lane == 0 ? g : inv[0]);   // lane 0: -gamma^2; others: beta
-    den = __shfl_sync(0xffffffffu, fma(m, inv[1], dl), 0);
-    beta = __shfl_sync(0xffffffffu, m, 1);
-  }
-  const double rr = __shfl_sync(0xffffffffu, v, 2);
-  ScalarRest q;
-  q.den = den;
+  const double dl = flow_total(2, G, sh);
+  const double den = k > 0 ? fma(q.m, q.inv_ga, dl) : dl;
   double alpha;
-  int st = -1;
-  if (moderate(den) && moderate(g)) {
-    const double a = lane == 2 ? g : den;
-    const double y0 = reciprocal_seed(a);
-    const double t1 = fma(lane == 0 ? g : -a, y0, lane == 0 ? 0.0 : 1.0);          // q0; 1 - a y0
-    if (!finite_bits(rr)) st = CGP_ERR_NONFINITE;
-    else if (nonneg_le(rr, sh.sc[4])) st = CGP_OK;   // (r,r) and (tol |b|)^2 are >= 0
-    else if (last) st = CGP_ERR_NOT_CONVERGED;
-    q.t = fma(lane == 0 ? -den : t1, lane == 0 ? t1 : y0, lane == 0 ? g : y0);     // g - den q0; y1
-    const double y1 = __shfl_sync(0xffffffffu, q.t, 1);
-    q.e = fma(lane == 0 ? q.t : -a, lane == 0 ? y1 : q.t, lane == 0 ? t1 : 1.0);   // alpha; 1 - a y1
-    alpha = q.e;
+  int st = q.st;
+  if (moderate(den) && moderate(q.g)) {
+    const double y0 = reciprocal_seed(den);
+    const double t1 = fma(lane == 0 ? q.g : -den, y0, lane == 0 ? 0.0 : 1.0);                   // q0; 1 - den y0
+    const double t2 = fma(lane == 0 ? -den : t1, lane == 0 ? t1 : y0, lane == 0 ? q.g : y0);    // g - den q0; y1
+    alpha = fma(t2, __shfl_sync(0xffffffffu, t2, 1), t1);                                       // lane 0: q0 + rem y1
   } else {
-    if (!finite_bits(g) || !finite_bits(dl) || !finite_bits(rr)) st = CGP_ERR_NONFINITE;
-    else if (nonneg_le(rr, sh.sc[4])) st = CGP_OK;
-    else if (last) st = CGP_ERR_NOT_CONVERGED;
-    alpha = g / den;
-    q.t = 1.0 / g;
-    q.e = 0.0;
+    if (!finite_bits(dl)) st = CGP_ERR_NONFINITE;
+    alpha = q.g / den;
   }
   if (lane == 0) {
-    if (st < 0 && !(positive_bits(g) && positive_bits(alpha) && finite_bits(alpha))) st = CGP_ERR_BREAKDOWN;
+    if (st < 0 && !(positive_bits(q.g) && positive_bits(alpha) && finite_bits(alpha))) st = CGP_ERR_BREAKDOWN;
     sh.isc[0] = st;
-    sh.ab[k & 1][0] = alpha;
-    sh.ab[k & 1][1] = beta;
-    sh.sc[5] = rr;
+    sh.ea[k & 1] = alpha;
   }
-  return q;
-}
-// 1 / gamma (lane 2) and 1 / (gamma alpha) = den / gamma^2 on every lane.
-__device__ __forceinline__ void flow_scalars_rest(const ScalarRest& q, double (&inv)[2]) {
-  inv[0] = __shfl_sync(0xffffffffu, fma(q.e, q.t, q.t), 2);
-  inv[1] = q.den * inv[0] * inv[0];
+  q.den = den;
 }
 
 // Word of row j's w in the publication of reduction `red`.
@@ -337,15 +352,14 @@ __device__ __forceinline__ ulonglong2* flow_w64(const Desc& d, int red, int j) {
 //
 // Roles (a block has at least eight warps): the first half (ct threads) holds
 // the rows; four warps with an operation always ready fill the FP64 pipe, so
-// eight lose nothing in the product and halve the integer work of the partial
-// sums.  The other half folds and stores the partial sums, fetches the halo's
-// w, polls, derives the scalars and updates the ghost rows.  Keeping the rows'
-// r, s, w, u in registers (four rows a thread) was slower: 7.4 us an iteration.
+// eight lose nothing in the product.  The other half sums and stores the early
+// words, polls, fetches the halo's w, derives the scalars and updates the ghost
+// rows, each on warps of its own.  Keeping the rows' r, s, w, u in registers (four rows a thread) was
+// slower: 7.4 against 6.3 us an iteration.
 //
 // Measured at 512x256 on 152 blocks in O-grid tiles: 6.83 us an iteration with
-// the counter barrier and slots 16 bytes apart, 6.34 us in this form.  About
-// 4.5k of its 13.1k clocks are the product and the dot products on the FP64 pipe,
-// 1.3k the recurrences, 2.5k the exchange up to the last share, 1.7k the scalars.
+// the counter barrier and slots 16 bytes apart, 6.34 us with all sums after the
+// product, 5.59 us in this form.
 constexpr int kFlowMinBlock = 256;
 template <int T>
 __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
@@ -358,7 +372,13 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
   int red = 0;
   const int ow = nw / 2, ct = 32 * ow;                  // warps and threads with rows
   const int act = min(ow, (nloc * T + 31) / 32);        // of those, warps that have any
-  const int G = flow_groups(d.nblk, nw - ow);           // warps ow .. ow + G - 1 poll
+  const int G = flow_groups(d.nblk, nw - ow - 2);       // warps ow .. ow + G - 1 poll, warp ow + G derives the scalars
+  // With many rows the product outlasts the early words by far: the warps that
+  // poll for what it gives wait until this block's own part is done (866 rows:
+  // 5.72 -> 5.59 us an iteration, 745 rows: 6.98 -> 6.75 ms a solve).  With few
+  // rows the words are there almost at once and the wait costs a round trip (95
+  // rows: 1.23 -> 1.34 ms, 346 rows: 3.73 -> 3.81 ms).
+  const bool patient = chunk >= 512;
   double* const R0 = d.pub64 + 4 * n;                // r of a pass's start, for the ghost rows
   int* const mark = reinterpret_cast<int*>(d.z);     // rows that another block reads
 
@@ -421,10 +441,7 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
   };
   // this block's words start empty, its rows unmarked; the barrier of the first
   // reduction orders that before any block polls or marks
-  if (tid < 2) {
-    const uint64_t none[4] = {0, 0, 0, 0};
-    st_relaxed_v4(flow_line(d, tid, lb), none);
-  }
+  if (tid < 8) st_relaxed_b128(flow_line(d, tid / 4, tid / 2, lb) + 16 * (tid % 2), 0ull, 0ull);   // both kinds and banks
   for (int i = tid; i < nloc; i += bd) {
     *flow_w64(d, 0, r0 + i) = make_ulonglong2(0ull, 0ull);
     *flow_w64(d, 1, r0 + i) = make_ulonglong2(0ull, 0ull);
@@ -469,9 +486,11 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
     return;
   }
   const double stop = d.tol * bnorm, stop2 = stop * stop;
+  if (tid < 2) signal_init(&sh.sig[tid]);   // the barriers of the next passes order that before any use
   if (tid == 0) sh.sc[4] = stop2;   // the test ||r||^2 <= (tol ||b||)^2 needs no square root
 
   int its = 0, restarts = 0, status = CGP_ERR_NOT_CONVERGED, pending = -1;
+  unsigned phase = 0;   // of the block's signals, one of each an iteration
   double rr_rec = 0.0, rr_true = 0.0;
   bool first = true;
   while (true) {
@@ -503,87 +522,130 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
     first = false;
 
     // ---- u_0 and the ghost rows; then iterations from the product w_0 = K u_0 ----
-    for (int i = tid; i < nloc; i += bd) ext[own_at(i)] = ua[i];
     for (int h = tid; h < nh; h += bd) {
       const double rj = __ldcg(R0 + hid[h]);
       gr[h] = rj;
       ext[halo_at(h)] = dih[h] * rj;
     }
+    if (tid < ct) {
+      double g = 0.0, rr = 0.0;
+      for (int i = tid; i < nloc; i += ct) {
+        const double ri = r[i], ui = ua[i];
+        ext[own_at(i)] = ui;
+        g = fma(ri, ui, g);
+        rr = fma(ri, ri, rr);
+      }
+      sh.ev[0][tid] = g;
+      sh.ev[1][tid] = rr;
+    }
+    if (tid == 0) sh.tflag = 1;
     int k = 0;                           // products formed in this pass, less one
-    double inv[2] = {0.0, 0.0};          // the scalars' reciprocals (warp ow)
+    EarlyScalars es;                     // warp ow + G
+    es.inv_g = es.inv_ga = 0.0;
     while (true) {
       double* const uc = (k & 1) ? ub : ua;   // u_k
       double* const up = (k & 1) ? ua : ub;   // u_(k-1), then u_(k+1)
-      __syncthreads();
-      // ---- w_k = K u_k, published where another block reads it; the partial sums ----
-      double v3[3] = {0.0, 0.0, 0.0};
       const unsigned long long tag = (unsigned long long)red + 1;
+      __syncthreads();
       if (tid < ct) {
+        // ---- w_k = K u_k, published where another block reads it; (w,u) ----
+        double v = 0.0;
         rows(tid, ct, [&](int il, double sum) {
-          const double ui = uc[il], ri = r[il];
+          const double ui = uc[il];
           const bool out = pub[il];
           w[il] = sum;
-          v3[0] = fma(ri, ui, v3[0]);
-          v3[1] = fma(sum, ui, v3[1]);
-          v3[2] = fma(ri, ri, v3[2]);
+          v = fma(sum, ui, v);
           if (out) st_relaxed_b128(flow_w64(d, red, r0 + il), fx::dbits(sum), tag);
         });
-      }
-      flow_put(d, lb, red, act, ow, v3, sh);
-      // ---- p_(k-1) = u_(k-1) + beta p_(k-2), x += alpha p_(k-1) while the words travel ----
-      if (k > 0 && tid < ct) {
-        const double alpha = sh.ab[(k - 1) & 1][0], beta = sh.ab[(k - 1) & 1][1];
-        for (int i = tid; i < nloc; i += ct) {
-          const double pi = k == 1 ? up[i] : fma(beta, p[i], up[i]);
-          p[i] = pi;
-          x[i] = fma(alpha, pi, x[i]);
+        if (warp < act) flow_warp_sum(v, 2, warp, sh);
+        named_sync(2, ct);
+        if (warp == 0) {
+          flow_block_sum(2, act, flow_line(d, 1, red, lb), red, sh);
+          if (tid == 0) signal_give(&sh.sig[1]);
         }
-      }
-      // ---- the halo's w, then the records ----
-      ScalarRest rest;
-      if (warp >= ow) {
-        PollLimit lim(d);
-        constexpr int B = 4;   // loads of a thread in flight
-        const int nt = bd - ct;
-        for (int h = bd - 1 - tid; h < nh; h += B * nt) {   // the last warps first: they do not poll
-          ulonglong2 a[B];
-#pragma unroll
-          for (int q = 0; q < B; ++q)
-            a[q] = h + q * nt < nh ? ld_relaxed_b128(flow_w64(d, red, hid[h + q * nt])) : make_ulonglong2(0ull, tag);
-#pragma unroll
-          for (int q = 0; q < B; ++q) {
-            while (a[q].y != tag && !lim.expired()) a[q] = ld_relaxed_b128(flow_w64(d, red, hid[h + q * nt]));
-            if (a[q].y != tag) sh.tflag = 0;
-            if (h + q * nt < nh) gw[h + q * nt] = fx::from_bits(a[q].x);
+        // ---- p_(k-1) = u_(k-1) + beta p_(k-2), x += alpha p_(k-1) while the word travels ----
+        if (k > 0) {
+          const double alpha = sh.ea[(k - 1) & 1], beta = sh.eb[(k - 1) & 1];
+          for (int i = tid; i < nloc; i += ct) {
+            const double pi = k == 1 ? up[i] : fma(beta, p[i], up[i]);
+            p[i] = pi;
+            x[i] = fma(alpha, pi, x[i]);
           }
         }
-        if (warp < ow + G) {
-          if (!flow_poll(d, red, warp - ow, G, sh)) sh.tflag = 0;
-          named_sync(1, 32 * G);
-          if (warp == ow) rest = flow_scalars(G, k, its + k >= d.max_it, inv, sh);
+        // ---- s_k = w_k + beta_k s_(k-1), once beta_k is known ----
+        if (!signal_wait(&sh.sig[0], phase, d)) sh.tflag = 0;
+        const double beta = sh.eb[k & 1];
+        for (int i = tid; i < nloc; i += ct) s[i] = k == 0 ? w[i] : fma(beta, s[i], w[i]);
+      } else {
+        const int nt = bd - ct, cw = warp - ow;
+        // ---- the early words: (r,u) and (r,r) ----
+        if (cw < act) {
+          flow_warp_sum(sh.ev[0][tid - ct], 0, cw, sh);
+          flow_warp_sum(sh.ev[1][tid - ct], 1, cw, sh);
+        }
+        named_sync(3, nt);
+        if (warp >= nw - 2) {   // two warps that do not poll
+          const int c = warp - (nw - 2);
+          flow_block_sum(c, act, flow_line(d, 0, red, lb) + 16 * c, red, sh);
+        }
+        if (cw < G) {
+          ulonglong2 late = make_ulonglong2(0ull, 0ull);
+          if (!flow_poll<2>(d, 0, red, cw, G, 0, late, sh)) sh.tflag = 0;
+          named_sync(1, 32 * (G + 1));
+          if (patient && !signal_wait(&sh.sig[1], phase, d)) sh.tflag = 0;
+          if (!flow_poll<1>(d, 1, red, cw, G, 2, late, sh)) sh.tflag = 0;
+          named_sync(1, 32 * (G + 1));
+        } else if (cw == G) {
+          named_sync(1, 32 * (G + 1));
+          flow_early(es, G, k, its + k >= d.max_it, sh);
+          named_sync(1, 32 * (G + 1));
+          flow_late(es, G, k, sh);
+        } else {
+          // ---- the halo's w: other blocks store theirs about when this one does ----
+          if (patient && !signal_wait(&sh.sig[1], phase, d)) sh.tflag = 0;
+          PollLimit lim(d);
+          constexpr int B = 4;   // loads of a thread in flight
+          const int ht = nt - 32 * (G + 1);
+          for (int h = bd - 1 - tid; h < nh; h += B * ht) {
+            ulonglong2 a[B];
+#pragma unroll
+            for (int q = 0; q < B; ++q)
+              a[q] = h + q * ht < nh ? ld_relaxed_b128(flow_w64(d, red, hid[h + q * ht])) : make_ulonglong2(0ull, tag);
+#pragma unroll
+            for (int q = 0; q < B; ++q) {
+              while (a[q].y != tag && !lim.expired()) a[q] = ld_relaxed_b128(flow_w64(d, red, hid[h + q * ht]));
+              if (a[q].y != tag) sh.tflag = 0;
+              if (h + q * ht < nh) gw[h + q * ht] = fx::from_bits(a[q].x);
+            }
+          }
         }
       }
       __syncthreads();
       if (!sh.tflag) return;
       ++red;
+      phase ^= 1u;
       const int stop_st = sh.isc[0];
       if (stop_st >= 0) {
         if (stop_st != CGP_OK) pending = stop_st;
         break;
       }
-      const double alpha = sh.ab[k & 1][0], beta = sh.ab[k & 1][1];
-      // ---- own rows and ghost rows: s, r, u_(k+1) ----
+      const double alpha = sh.ea[k & 1], beta = sh.eb[k & 1];
       if (tid < ct) {
+        // ---- own rows: r, u_(k+1) and their dot products ----
+        double g = 0.0, rr = 0.0;
         for (int i = tid; i < nloc; i += ct) {
-          const double si = k == 0 ? w[i] : fma(beta, s[i], w[i]);
-          s[i] = si;
-          const double ri = fma(-alpha, si, r[i]);
+          const double ri = fma(-alpha, s[i], r[i]);
           r[i] = ri;
           const double ui = di[i] * ri;
           up[i] = ui;
           ext[own_at(i)] = ui;
+          g = fma(ri, ui, g);
+          rr = fma(ri, ri, rr);
         }
+        sh.ev[0][tid] = g;
+        sh.ev[1][tid] = rr;
       } else {
+        // ---- ghost rows: s, r, u_(k+1) ----
         for (int h = bd - 1 - tid; h < nh; h += bd - ct) {
           const double sj = k == 0 ? gw[h] : fma(beta, gs[h], gw[h]);
           gs[h] = sj;
@@ -591,7 +653,7 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
           gr[h] = rj;
           ext[halo_at(h)] = dih[h] * rj;
         }
-        if (warp == ow) flow_scalars_rest(rest, inv);
+        if (warp == ow + G) es.inv_ga = es.den * es.inv_g * es.inv_g;   // 1 / (gamma alpha) = den / gamma^2
       }
       ++k;
     }
@@ -640,7 +702,7 @@ __device__ __forceinline__ void flow_put_f(const Desc& d, int lb, int red, int a
       for (int o = 8; o > 0; o >>= 1) t[c] += __shfl_xor_sync(0xffffffffu, t[c], o);   // at most 16 warps
     }
     if (lane == 0)
-      st_relaxed_b128(flow_line(d, red, lb),
+      st_relaxed_b128(flow_line(d, 0, red, lb),
                       ((unsigned long long)__float_as_uint(t[1]) << 32) | __float_as_uint(t[0]),
                       ((unsigned long long)(unsigned)(red + 1) << 32) | __float_as_uint(t[2]));
   }
@@ -656,7 +718,7 @@ __device__ __forceinline__ bool flow_poll_f(const Desc& d, int red, int q, int G
   float acc[3] = {0.0f, 0.0f, 0.0f};
   for (int base = 32 * q; base < d.nblk; base += 32 * G) {
     const int j = base + lane;
-    const void* line = flow_line(d, red, j < d.nblk ? j : base);
+    const void* line = flow_line(d, 0, red, j < d.nblk ? j : base);
     ulonglong2 a;
     while (true) {
       a = ld_relaxed_b128(line);
@@ -726,6 +788,9 @@ __device__ __forceinline__ unsigned long long* flow_w32(const Desc& d, int red, 
 // on from the shared-memory slice.  R = 0 keeps everything in shared memory.
 // At 512x256 on 152 blocks an inner iteration takes 2.55 us (3.69 us with the
 // counter barrier), at 64x32 on 9 blocks 2.0 us (4.0 us).
+//
+// The sums go out together after the product: its 0.8k clocks are too few to
+// hide a second exchange (early and late words as in solve_fp64_flow: 2.82 us).
 template <int T, int R>
 __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -798,7 +863,7 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
 
   // this block's words start empty, its rows unmarked; the barrier of the first
   // reduction orders that before any block polls or marks
-  if (tid < 2) st_relaxed_b128(flow_line(d, tid, lb), 0ull, 0ull);
+  if (tid < 2) st_relaxed_b128(flow_line(d, 0, tid, lb), 0ull, 0ull);
   for (int i = tid; i < nloc; i += bd) {
     *flow_w32(d, 0, r0 + i) = 0ull;
     *flow_w32(d, 1, r0 + i) = 0ull;

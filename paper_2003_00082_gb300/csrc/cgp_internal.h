@@ -148,7 +148,7 @@ struct cgp_mesh_impl {
   float* f32own = nullptr;   // [6 n] mixed without shared-memory residency: own inner vectors
   float* fpart = nullptr;    // [8 * max_blocks] FP32 partial sums
   double* part = nullptr;    // [max_blocks * 32] per-block fixed-point partial sums
-  unsigned long long* tpart = nullptr;  // [max_blocks][2] lines of kLineBytes: tagged partial sums by bank
+  unsigned long long* tpart = nullptr;  // [max_blocks][4] lines of kLineBytes: tagged partial sums by kind and bank
   unsigned* nflag = nullptr; // [max_blocks] pipelined tiles: published-w counts of the blocks
   unsigned* bar = nullptr;   // grid barrier counter
   SolveResult* res = nullptr;

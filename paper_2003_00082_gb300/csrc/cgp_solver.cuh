@@ -107,13 +107,16 @@ struct Shared {
   float fsc[8];
   int flag;
   int tflag;                    // outcome of the last tagged reduction's wait
-  long long phi[3][8];          // dataflow iterations: the polling warps' shares of the totals
+  // dataflow iterations: the polling warps' shares of the totals; alpha and beta by iteration
+  // parity; the FP64 rows' parts of (r,u) and (r,r); the signals beta ready
+  // and (w,u) stored
+  long long phi[3][8];
   int pexp[3][8];
   float pf[3][8];
-  long long bsum[3];            // ... the block's partial sums
-  int bexp[3];
-  double ab[2][2];              // ... alpha and beta by iteration parity
+  double ea[2], eb[2];
   float abf[2][2];
+  double ev[2][MAX_BLOCK / 2];
+  unsigned long long sig[2];
 };
 
 // Barrier over the blocks of one instance (cgp_sync.h): a block that gives
@@ -185,7 +188,7 @@ __device__ __forceinline__ unsigned long long* part_slot(const Desc& d, int red,
 // zeroes its slots at the start of a launch.
 __device__ __forceinline__ ulonglong2* tag_slot(const Desc& d, int red, int c, int blk) {
   return reinterpret_cast<ulonglong2*>(reinterpret_cast<unsigned char*>(d.tpart) +
-                                       ((size_t)blk * 2 + (red & 1)) * kLineBytes) + c;
+                                       ((size_t)blk * 4 + (red & 1)) * kLineBytes) + c;
 }
 
 // Sum NC (<= 3) per-thread values over the block; warp c then folds
@@ -1699,7 +1702,7 @@ __device__ void solve_fp64_pl(const Desc& d, int lb, Shared& sh) {
 // block zeroes its words at launch start).  Banks by the reduction's parity.
 __device__ __forceinline__ unsigned long long* ftag_slot(const Desc& d, int red, int c, int blk) {
   return reinterpret_cast<unsigned long long*>(reinterpret_cast<unsigned char*>(d.tpart) +
-                                               ((size_t)blk * 2 + (red & 1)) * kLineBytes) + c;
+                                               ((size_t)blk * 4 + (red & 1)) * kLineBytes) + c;
 }
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
