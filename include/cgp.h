@@ -475,10 +475,10 @@ int cgp_mesh_set_ogrid(cgp_mesh m, int n_theta, int n_r);
  *         SpMV: bit 0 uses the O-grid stencil form (cgp_mesh_set_ogrid) with
  *         one thread per row (lanes ignored).
  * All zero (as after cgp_assemble) lets the solver choose: tagged reductions
- * with rows in shared memory where they fit; FP64 about 96 rows per block, on
- * O-grid tiles (registered meshes) or, from 4096 rows on, in the bisection
- * order (the renumbered system is built by the first solve); MIXED about 256
- * rows per block.
+ * with rows in shared memory where they fit; FP64 about 96 rows per block (64
+ * below 2500 rows), on O-grid tiles (registered meshes) or, from 4096 rows on,
+ * in the bisection order (the renumbered system is built by the first solve);
+ * MIXED about 352 rows per block on at least 12 blocks.
  * Invalid shapes are rejected with INVALID_ARG.  cgp_autotune sets these.
  */
 typedef enum {

@@ -57,7 +57,9 @@ __global__ void __launch_bounds__(MAX_BLOCK) pcg_persistent_kernel(Desc d) {
 }
 
 // ---------------------------------------------------------------------------
-// standalone SpMV: T lanes per row, grid-stride over row groups
+// standalone SpMV: T lanes per row, grid-stride over row groups.  (Taking a row's
+// entries eight at a time with predicated loads was slower: 45 against 41 us in
+// FP64 at 2048x1024.)
 // ---------------------------------------------------------------------------
 template <int T, typename V>
 __global__ void __launch_bounds__(256) spmv_kernel(int n, const int* __restrict__ rowptr,
@@ -638,24 +640,30 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
 // shape used).  The dataflow iterations (flag bit 3) wherever rows fit in shared
 // memory, 512 threads a block.  FP64: about 96 rows a block, since the exchange
 // costs nearly the same for any number of blocks while the FP64 pipe of every SM
-// takes its share of the rows (128x64: 1.32 ms on 76 blocks, 1.99 ms on 35 with
-// 256 rows; 64x32: 0.60 ms on 24, 0.91 ms on 9); O-grid tiles where the mesh is
-// registered (512x256: 8.3 ms against 9.0 ms in the bisection order and 11.0 ms
-// in the mesh's own), else the bisection order from 4096 rows on (321x163: 4.0
-// against 4.4 ms), below which it gains nothing.  MIXED: 256 rows a block in the
-// mesh's order (64x32 0.43 ms with 9 blocks, 0.44 with 24; bisection gains under
-// 1 % at any size and costs a second copy of the system).  Systems whose rows do
-// not fit keep the barrier forms with rows in global memory.
+// takes its share of the rows (129x67: 1.24 ms on 92 blocks, 1.47 ms on 24);
+// O-grid tiles where the mesh is registered (512x256: 7.4 ms against 8.2 ms in the
+// bisection order and 10.2 ms in the mesh's own), else the bisection order from
+// 4096 rows on (321x163: 3.7 against 4.1 ms), below which it gains nothing.
+// MIXED: about 352 rows a block but at least 12 blocks, in the mesh's order: up to
+// about 12 blocks share one GPC, where the exchange is shortest (90x45: 0.60 ms on
+// 12 blocks, 0.69 ms on 17); bisection gains under 1 % at any size and costs a
+// second copy of the system.  Below 2500 rows a block has 256 threads, whose
+// barriers are cheaper (64x32: FP64 0.545 ms on 33 blocks of 256 threads, 0.567 ms
+// on 22 of 512; MIXED 0.42 and 0.44 ms on 12).  Systems whose rows do not fit keep
+// the barrier forms with rows in global memory.
 int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps, SolverTuning& tu) {
   const int n = m->n_c, sms = std::max(1, dev_info(m->device).sms);
-  const int rows = mixed ? 256 : 96;
-  const int nblk = std::min(sms, std::max(1, (n + rows - 1) / rows));
+  const bool small = n < 2500;
+  const int block = small ? 256 : 512;
+  const int few = (n + 63) / 64;   // blocks of 64 rows
+  int nblk = mixed ? (small ? std::min(12, few) : std::max(12, (n + 351) / 352)) : (small ? few : (n + 95) / 96);
+  nblk = std::min(sms, std::max(1, nblk));
   int flags[3], count = 0;
   if (!mixed && nblk > 1 && m->st_nt > 0) flags[count++] = 40;
   if (!mixed && n >= 4096) flags[count++] = 12;
   flags[count++] = 8;
   for (int k = 0; k < count; ++k) {
-    tu = SolverTuning{512, 1, nblk, flags[k]};
+    tu = SolverTuning{block, 1, nblk, flags[k]};
     // a renumbered system that cannot be allocated is no reason to refuse the solve
     if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.res) return CGP_OK;
   }
@@ -865,7 +873,8 @@ int launch_spmv(cgp_mesh_impl* m, int precision, const void* x, void* y, cudaStr
   const SolverTuning& tu = m->tune[precision == CGP_FP64 ? CGP_TUNE_SPMV_FP64 : CGP_TUNE_SPMV_FP32];
   if (tu.flags & 1) return launch_spmv_stencil(m, precision, x, y, tu.block, s);   // O-grid stencil form
   const int block = tu.block > 0 ? tu.block : 256;
-  const int lanes = tu.lanes > 0 ? tu.lanes : (precision == CGP_FP64 ? 1 : 4);
+  // one lane per row on the seven entries of a triangular mesh (FP32 at 2048x1024: 29 us, with four 52 us)
+  const int lanes = tu.lanes > 0 ? tu.lanes : 1;
   long long grid = tu.blocks;
   if (grid <= 0) {
     grid = ((long long)m->n_c * lanes + block - 1) / block;
@@ -900,8 +909,8 @@ __global__ void barrier_selftest_kernel(unsigned* bar, int* timeout, int nblk, i
 // Batched solves: many meshes, one persistent cooperative launch
 // ---------------------------------------------------------------------------
 struct BatchShape {
-  int block = 512;
-  int lanes = 1;
+  int block = 0;    // 0: 512
+  int lanes = 0;    // 0: 1
   int per_sm = 0;   // blocks per SM (0: as many as can be co-resident)
   int flags = 0;    // bit 0: rows in global memory; bit 1: classic FP64 iteration; bit 2: one packed launch
 };
