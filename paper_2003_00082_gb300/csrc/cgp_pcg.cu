@@ -650,8 +650,10 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
 // second copy of the system.  Below 2500 rows a block has 256 threads, whose
 // barriers are cheaper (64x32: FP64 0.545 ms on 33 blocks of 256 threads, 0.567 ms
 // on 22 of 512; MIXED 0.42 and 0.44 ms on 12).  Systems whose rows do not fit keep
-// the barrier forms with rows in global memory.
-int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps, SolverTuning& tu) {
+// the barrier forms with rows in global memory; so does a solve under stream
+// capture whose renumbered system or halo lists are not there yet, since building
+// them allocates and synchronises.
+int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps, SolverTuning& tu, cudaStream_t s) {
   const int n = m->n_c, sms = std::max(1, dev_info(m->device).sms);
   const bool small = n < 2500;
   const int block = small ? 256 : 512;
@@ -662,12 +664,23 @@ int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps,
   if (!mixed && nblk > 1 && m->st_nt > 0) flags[count++] = 40;
   if (!mixed && n >= 4096) flags[count++] = 12;
   flags[count++] = 8;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
+  const bool capturing = cap != cudaStreamCaptureStatusNone;
+  auto built = [&](int fl) {
+    if (!(fl & 36)) return std::any_of(m->plans.begin(), m->plans.end(), [&](const HaloPlan& p) { return p.nblk == nblk; });
+    const int dir = m->far_dirichlet ? 1 : 0, tiles = (fl & 32) ? 1 : 0;
+    return std::any_of(m->psys.begin(), m->psys.end(), [&](const PermSystem& p) {
+      return p.nblk == nblk && p.dirichlet == dir && p.tiles == tiles;
+    });
+  };
   for (int k = 0; k < count; ++k) {
+    if (capturing && !built(flags[k])) continue;
     tu = SolverTuning{block, 1, nblk, flags[k]};
     // a renumbered system that cannot be allocated is no reason to refuse the solve
     if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.res) return CGP_OK;
   }
-  tu = SolverTuning{0, 0, 0, 0};
+  tu = SolverTuning{0, 0, 0, capturing ? 1 : 0};
   return plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps);
 }
 
@@ -759,7 +772,7 @@ int launch_solve(cgp_mesh_impl* m, const double* b, double* x, const cgp_solve_o
   LaunchPlan plan;
   PermSystem* ps = nullptr;
   int st = tu.block == 0 && tu.lanes == 0 && tu.blocks == 0 && tu.flags == 0
-               ? plan_default(m, mixed, plan, &ps, tu)
+               ? plan_default(m, mixed, plan, &ps, tu, s)
                : plan_solve(m, m->device, m->n_c, m->max_blocks, tu, mixed, plan, &ps);
   if (st != CGP_OK) return st;
   const int nblk = plan.nblk;

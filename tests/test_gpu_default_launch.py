@@ -38,3 +38,28 @@ def test_default_launch_agrees_with_an_explicit_one(nt, nr, ogrid, far, precisio
     d = float(torch.linalg.norm(out[0] - out[1]) / torch.linalg.norm(out[1]))
     assert d <= 2e-11 * max(10.0, (nt / 2.0) ** 2), d
     m.close()
+
+
+@pytest.mark.parametrize("warm", [False, True])
+def test_untuned_solve_under_stream_capture(warm):
+    """A captured untuned solve replays to the same answer, whether or not a first solve has built its plan."""
+    from paper_2003_00082_gb300 import build, cgp
+    build.build()
+    cgp.load()
+    m = cgp.Mesh(*inputs.ogrid(129, 40))     # more than 4096 rows: the bisection order when it can be built
+    b = np.random.default_rng(3).standard_normal(m.n_c)
+    b = torch.as_tensor(b - b.mean(), device=DEV)
+    x, ref = torch.zeros_like(b), torch.zeros_like(b)
+    if warm:
+        cgp.cgp_poisson_solve(m.handle, b, x, tol=1e-11)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        cgp.cgp_poisson_solve_async(m.handle, b, x, tol=1e-11)
+    x.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert cgp.cgp_last_launch(m.handle)["resident"] == int(warm)
+    assert cgp.cgp_poisson_solve(m.handle, b, ref, tol=1e-11)["status"] == cgp.CGP_OK
+    assert float(torch.linalg.norm(x - ref) / torch.linalg.norm(ref)) <= 2e-11 * (129 / 2.0) ** 2
+    m.close()
