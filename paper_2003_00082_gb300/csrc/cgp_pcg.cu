@@ -1648,7 +1648,7 @@ extern "C" int cgp_autotune(cgp_mesh m, int precision, const double* b, double* 
   cgp_solve_opts o{1e-8, 20000, precision, 1e-4, 0, 50};
   const int sms = std::max(1, dev_info(m->device).sms);
   std::vector<int> counts;
-  if (m->n_c <= 16384) counts = {1, 2, 4, 8, 16};
+  if (m->n_c <= 16384) counts = {1, 2, 4, 8, 12, 16, 32};
   for (int c : {sms / 2, sms, 2 * sms})
     if (c >= 1 && c <= m->n_c / 32) counts.push_back(c);
   if (counts.empty()) counts.push_back(1);
