@@ -497,7 +497,7 @@ int cgp_get_tuning(cgp_mesh m, int what, int* block, int* lanes, int* blocks, in
  * Runs the solve (precision CGP_FP64 or CGP_MIXED, tol 1e-8, from x = 0) on
  * the caller's right-hand side b (device [n_c]) for every candidate of
  * threads per block {256, 512}, lanes per CSR row {1, 2, 4}, grid size (a
- * few counts around the SM count, and 1..16 blocks for small systems),
+ * few counts around the SM count, and 1..32 blocks for small systems),
  * shared-memory residency, the row order (flag bit 2), the reduction form
  * (flag bit 3) and, for FP64, the iteration form (flag bits 1 and 4) and,
  * on meshes registered with cgp_mesh_set_ogrid, the O-grid tiles with the
