@@ -5,6 +5,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -177,6 +178,7 @@ struct cgp_mesh_impl {
   int* vop_col = nullptr;         // [vop_off's last]
   double* vop_coef = nullptr;     // [vop_off's last][2] weights of the mean gradient's x and y
   void* vop_base = nullptr;
+  std::mutex vop_mu;              // held while the operator is looked up or built
 
   std::vector<HaloPlan> plans;   // cached per block count
   std::vector<PermSystem> psys;  // cached per (block count, boundary condition, tiles)

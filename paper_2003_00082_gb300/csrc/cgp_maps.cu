@@ -329,8 +329,10 @@ int launch_parent_shape(cgp_mesh_impl* m, cudaStream_t s) {
 }
 
 // The velocity correction's operator, built once per mesh: the incidence lists
-// on the host, the rows on the GPU.
+// on the host, the rows on the GPU.  The map calls share no scratch, so several
+// host threads may make them on one mesh: one of them builds, the others wait.
 static int build_correction(cgp_mesh_impl* m, cudaStream_t s) {
+  std::lock_guard<std::mutex> lk(m->vop_mu);
   if (m->vop_base) return CGP_OK;
   const std::vector<int>& tp = m->levels >= 2 ? m->h_tri_par : m->h_tri_c;
   const std::vector<int>& mp = m->levels >= 2 ? m->h_mid_par : m->h_tri_mid;

@@ -39,3 +39,27 @@ def test_velocity_correction_around_a_hub(spokes):
     for got, old, ref in zip(out, (u, v), O.velocity_correct(om.xy_f, om.tri_f, p, u, v, 0.05)):
         assert np.linalg.norm(got.cpu().numpy() - ref) <= 3e-16 * spokes * np.linalg.norm(ref - old) + 1e-15 * np.linalg.norm(ref)
     m.close()
+
+
+def test_first_corrections_of_several_threads():
+    """Host threads that make the first velocity correction on one mesh at the same time, each on its own stream: one
+    builds the operator, and all get the bits of a later call."""
+    from concurrent.futures import ThreadPoolExecutor
+
+    from paper_2003_00082_gb300 import build, cgp, inputs
+    build.build()
+    cgp.load()
+    m = cgp.Mesh(*inputs.ogrid(129, 40))
+    rng = np.random.default_rng(3)
+    p, u, v = (T(rng.standard_normal(m.n_f)) for _ in range(3))
+    jobs = [(torch.cuda.Stream(), torch.empty_like(u), torch.empty_like(v)) for _ in range(4)]
+    torch.cuda.synchronize()
+    with ThreadPoolExecutor(4) as ex:
+        list(ex.map(lambda j: cgp.cgp_velocity_correct(m.handle, p, u, v, 0.05, j[1], j[2], stream=j[0]), jobs))
+    torch.cuda.synchronize()
+    ref = torch.empty_like(u), torch.empty_like(v)
+    cgp.cgp_velocity_correct(m.handle, p, u, v, 0.05, *ref)
+    torch.cuda.synchronize()
+    for _, a, b in jobs:
+        assert torch.equal(a, ref[0]) and torch.equal(b, ref[1])
+    m.close()
