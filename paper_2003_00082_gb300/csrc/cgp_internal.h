@@ -101,6 +101,11 @@ struct PermSystem {
   void* st_base = nullptr;
 };
 
+// A launch that the default rule found not to work on a mesh.
+struct RejectedLaunch {
+  int nblk, dirichlet, flags, mixed;
+};
+
 struct cgp_mesh_impl {
   int device = 0;
   int n_c = 0, t_c = 0, n_e = 0, n_f = 0, t_f = 0, nnz = 0;
@@ -182,6 +187,7 @@ struct cgp_mesh_impl {
 
   std::vector<HaloPlan> plans;   // cached per block count
   std::vector<PermSystem> psys;  // cached per (block count, boundary condition, tiles)
+  std::vector<RejectedLaunch> rejected;
   SolverTuning tune[4] = {{0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}, {0, 0, 0, 0}};  // by cgp_tune_target
   PlanRecord last_plan[2] = {{0, 0, 0, 0}, {0, 0, 0, 0}};                          // FP64, MIXED
 };

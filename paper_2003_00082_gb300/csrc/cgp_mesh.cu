@@ -24,7 +24,10 @@ int fail(int status, const std::string& msg) {
   return status;
 }
 
+// A failed call also stays behind as the thread's last CUDA error, where the
+// next kernel launch's check would find it: it is reported here and taken back.
 int cuda_fail(cudaError_t e, const char* what) {
+  cudaGetLastError();
   std::string m = std::string(what) + ": " + cudaGetErrorName(e) + " (" + cudaGetErrorString(e) + ")";
   return fail(e == cudaErrorMemoryAllocation ? CGP_ERR_OOM : CGP_ERR_CUDA, m);
 }

@@ -652,7 +652,10 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
 // on 22 of 512; MIXED 0.42 and 0.44 ms on 12).  Systems whose rows do not fit keep
 // the barrier forms with rows in global memory; so does a solve under stream
 // capture whose renumbered system or halo lists are not there yet, since building
-// them allocates and synchronises.
+// them allocates and synchronises.  A form that does not fit, or whose system
+// cannot be allocated, is no reason to refuse the solve: the next one is taken,
+// and the mesh remembers it, so that later solves do not try (and synchronise)
+// again.
 int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps, SolverTuning& tu, cudaStream_t s) {
   const int n = m->n_c, sms = std::max(1, dev_info(m->device).sms);
   const bool small = n < 2500;
@@ -667,18 +670,24 @@ int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps,
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) cudaGetLastError();
   const bool capturing = cap != cudaStreamCaptureStatusNone;
+  const int dir = m->far_dirichlet ? 1 : 0, mx = mixed ? 1 : 0;
   auto built = [&](int fl) {
     if (!(fl & 36)) return std::any_of(m->plans.begin(), m->plans.end(), [&](const HaloPlan& p) { return p.nblk == nblk; });
-    const int dir = m->far_dirichlet ? 1 : 0, tiles = (fl & 32) ? 1 : 0;
+    const int tiles = (fl & 32) ? 1 : 0;
     return std::any_of(m->psys.begin(), m->psys.end(), [&](const PermSystem& p) {
       return p.nblk == nblk && p.dirichlet == dir && p.tiles == tiles;
     });
   };
+  auto rejected = [&](int fl) {
+    return std::any_of(m->rejected.begin(), m->rejected.end(), [&](const RejectedLaunch& r) {
+      return r.nblk == nblk && r.dirichlet == dir && r.flags == fl && r.mixed == mx;
+    });
+  };
   for (int k = 0; k < count; ++k) {
-    if (capturing && !built(flags[k])) continue;
+    if (rejected(flags[k]) || (capturing && !built(flags[k]))) continue;
     tu = SolverTuning{block, 1, nblk, flags[k]};
-    // a renumbered system that cannot be allocated is no reason to refuse the solve
     if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.res) return CGP_OK;
+    if (!capturing) m->rejected.push_back(RejectedLaunch{nblk, dir, flags[k], mx});
   }
   tu = SolverTuning{0, 0, 0, capturing ? 1 : 0};
   return plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps);
