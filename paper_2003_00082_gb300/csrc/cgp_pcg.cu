@@ -636,6 +636,35 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
   return CGP_OK;
 }
 
+// Dynamic shared memory that a block of `fn` may ask for.
+size_t smem_limit(const void* fn, int device) {
+  cudaFuncAttributes fa{};
+  if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (size_t)std::max(0, optin_smem(device) - (int)fa.sharedSizeBytes - 1024);
+}
+
+// Whether the rows of a renumbered FP64 launch can be resident at all: what its
+// largest block needs without any halo (it holds no fewer entries than the mean).
+// Asked before the system is built, which takes host work, a synchronisation and
+// a second copy of the system on the device (1024x512: 124 MiB in tiles, 92 MiB
+// in the bisection order).
+bool renumbered_rows_can_fit(const cgp_mesh_impl* m, int nblk, int block, bool tiles) {
+  const int chunk = (m->n_c + nblk - 1) / nblk, nnz = (m->nnz + nblk - 1) / nblk;
+  SolverKind kind = KIND_FP64_SR;
+  const PcgFn fn = resident_kernel_for(kind, 1, block);
+  const size_t need = tiles ? res_smem_stencil(chunk, 0, chunk) : res_smem_rows(kind, chunk, nnz);
+  return need <= smem_limit((const void*)fn, m->device);
+}
+
+void free_perm_system(PermSystem& ps) {
+  cudaFree(ps.base);
+  cudaFree(ps.plan.base);
+  cudaFree(ps.st_base);
+}
+
 // Launch of a mesh that was never tuned (tuning all zero; `tu` receives the
 // shape used).  The dataflow iterations (flag bit 3) wherever rows fit in shared
 // memory, 512 threads a block.  FP64: about 96 rows a block, since the exchange
@@ -685,8 +714,15 @@ int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps,
   };
   for (int k = 0; k < count; ++k) {
     if (rejected(flags[k]) || (capturing && !built(flags[k]))) continue;
-    tu = SolverTuning{block, 1, nblk, flags[k]};
-    if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.res) return CGP_OK;
+    const size_t systems = m->psys.size();
+    if (built(flags[k]) || !(flags[k] & 36) || renumbered_rows_can_fit(m, nblk, block, (flags[k] & 32) != 0)) {
+      tu = SolverTuning{block, 1, nblk, flags[k]};
+      if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.res) return CGP_OK;
+    }
+    if (m->psys.size() > systems) {   // built here, and its halo was too much
+      free_perm_system(m->psys.back());
+      m->psys.pop_back();
+    }
     if (!capturing) m->rejected.push_back(RejectedLaunch{nblk, dir, flags[k], mx});
   }
   tu = SolverTuning{0, 0, 0, capturing ? 1 : 0};

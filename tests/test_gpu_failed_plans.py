@@ -68,3 +68,27 @@ def test_renumbered_system_that_does_not_fit_the_memory():
     assert torch.equal(x, x2)
     m.close()
     small.close()
+
+
+@pytest.mark.parametrize("ogrid", [False, True])
+@pytest.mark.parametrize("nt,nr", [(1024, 512), (690, 340), (676, 336), (640, 310), (634, 306)])
+def test_systems_too_large_for_shared_memory_are_not_copied(nt, nr, ogrid):
+    """Rows that cannot be resident (far beyond the limit, and a few percent around it, where only the halo decides):
+    the first solve leaves no renumbered copy behind, at most the halo lists (4 bytes an entry and the lists)."""
+    from paper_2003_00082_gb300 import build, cgp
+    build.build()
+    cgp.load()
+    m = cgp.Mesh(*inputs.ogrid(nt, nr))
+    if ogrid:
+        cgp.cgp_mesh_set_ogrid(m.handle, nt, nr)
+    b = torch.as_tensor(np.random.default_rng(4).standard_normal(m.n_c), device=DEV)
+    b -= b.mean()
+    x = torch.zeros_like(b)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    assert cgp.cgp_poisson_solve(m.handle, b, x)["status"] == cgp.CGP_OK
+    if not cgp.cgp_last_launch(m.handle)["resident"]:
+        assert free - torch.cuda.mem_get_info()[0] <= 8 * m.nnz + 4 * MB
+    else:
+        assert m.n_c < 245000
+    m.close()
