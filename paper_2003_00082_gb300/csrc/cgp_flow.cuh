@@ -43,7 +43,29 @@
 namespace cgp {
 namespace {
 
-constexpr int kMaxShares = 8;   // groups of blocks whose records are folded by one warp each
+constexpr int kMaxShares = 8;   // groups of blocks whose words are folded by one warp each
+
+// What only the dataflow iterations keep in shared memory beside Shared: it leads
+// the dynamic part, so that the other forms' blocks stay as small as they are
+// (whole 16-byte units; flow_smem_bytes counts them).
+struct Flow64Shared {
+  long long phi[3][kMaxShares];   // the polling warps' shares of the totals
+  int pexp[3][kMaxShares];
+  double ea[2], eb[2];            // alpha and beta by iteration parity
+  double ev[2][MAX_BLOCK / 2];    // the rows' parts of (r,u) and (r,r)
+  unsigned long long sig[2];      // signals: beta ready, (w,u) stored
+};
+struct Flow32Shared {
+  float pf[3][kMaxShares];        // the polling warps' shares of the totals
+  float abf[2][2];                // alpha and beta by iteration parity
+};
+static_assert(sizeof(Flow64Shared) % 16 == 0 && sizeof(Flow32Shared) % 16 == 0, "the vectors that follow are aligned");
+
+// Dynamic shared memory of a dataflow block of `chunk` rows beyond the barrier
+// form's: the state above and a byte per row (published or not).
+inline size_t flow_smem_bytes(bool mixed, int chunk) {
+  return (mixed ? sizeof(Flow32Shared) : sizeof(Flow64Shared)) + ((size_t)chunk + 15) / 16 * 16;
+}
 
 // A block's line of bank (red & 1): kind 0 early words, 1 the late word.
 __device__ __forceinline__ unsigned char* flow_line(const Desc& d, int kind, int red, int blk) {
@@ -183,7 +205,7 @@ __device__ __forceinline__ void flow_block_sum(int c, int act, void* p, int red,
 }
 
 // Polling warp q < G: wait for NC words of kind `kind` of the blocks 32 q + lane
-// (+ 32 G ...); the warp's shares of the totals go to sh.phi/pexp[c0 + c][q],
+// (+ 32 G ...); the warp's shares of the totals go to fs.phi/pexp[c0 + c][q],
 // value phi 2^(pexp - 1074), |phi| < 2^62.  A block's partial enters with 57
 // bits relative to the largest one.  The warp that has the early words (kind 0)
 // loads its late word at once, into `late`, so that the load travels while the
@@ -191,7 +213,7 @@ __device__ __forceinline__ void flow_block_sum(int c, int act, void* p, int red,
 // `late`.  False (on every lane) when the wait gave up.
 template <int NC>
 __device__ __forceinline__ bool flow_poll(const Desc& d, int kind, int red, int q, int G, int c0, ulonglong2& late,
-                                          Shared& sh) {
+                                          Flow64Shared& fs) {
   const int lane = threadIdx.x & 31;
   PollLimit lim(d);
   const unsigned tag = (unsigned)(red + 1);
@@ -243,8 +265,8 @@ __device__ __forceinline__ bool flow_poll(const Desc& d, int kind, int red, int 
     }
   }
   if (lane < NC) {
-    sh.phi[c0 + lane][q] = NC == 2 && lane == 1 ? acc[NC - 1] : acc[0];
-    sh.pexp[c0 + lane][q] = NC == 2 && lane == 1 ? Ea[NC - 1] : Ea[0];
+    fs.phi[c0 + lane][q] = NC == 2 && lane == 1 ? acc[NC - 1] : acc[0];
+    fs.pexp[c0 + lane][q] = NC == 2 && lane == 1 ? Ea[NC - 1] : Ea[0];
   }
   return true;
 }
@@ -259,10 +281,10 @@ __device__ __forceinline__ double scaled_double(long long X, int E) {
 }
 
 // One warp: the total of component c from its G shares, on every lane.
-__device__ __forceinline__ double flow_total(int c, int G, const Shared& sh) {
+__device__ __forceinline__ double flow_total(int c, int G, const Flow64Shared& fs) {
   const int lane = threadIdx.x & 31;
-  const long long x = lane < G ? sh.phi[c][lane] : 0ll;
-  const int e = lane < G ? sh.pexp[c][lane] : 1;
+  const long long x = lane < G ? fs.phi[c][lane] : 0ll;
+  const int e = lane < G ? fs.pexp[c][lane] : 1;
   const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
   const long long X = warp_sum57(E < fx::kBadExp ? (x >> min(E - e + 3, 63)) : 0ll);   // eight shares of 59 bits
   return scaled_double(X, E + 3);
@@ -299,15 +321,15 @@ struct EarlyScalars {
   double den;              // denominator of alpha
   int st;                  // stop status so far (-1: go on)
 };
-// Leaves beta in sh.eb[k & 1] and gives sig[0] once it is there.
-__device__ __forceinline__ void flow_early(EarlyScalars& q, int G, int k, bool last, Shared& sh) {
-  q.g = flow_total(0, G, sh);
+// Leaves beta in fs.eb[k & 1] and gives sig[0] once it is there.
+__device__ __forceinline__ void flow_early(EarlyScalars& q, int G, int k, bool last, Flow64Shared& fs, Shared& sh) {
+  q.g = flow_total(0, G, fs);
   const double beta = k > 0 ? q.g * q.inv_g : 0.0;
   if ((threadIdx.x & 31) == 0) {
-    sh.eb[k & 1] = beta;
-    signal_give(&sh.sig[0]);
+    fs.eb[k & 1] = beta;
+    signal_give(&fs.sig[0]);
   }
-  q.rr = flow_total(1, G, sh);
+  q.rr = flow_total(1, G, fs);
   q.st = -1;
   if (!finite_bits(q.g) || !finite_bits(q.rr)) q.st = CGP_ERR_NONFINITE;
   else if (nonneg_le(q.rr, sh.sc[4])) q.st = CGP_OK;   // (r,r) and (tol |b|)^2 are >= 0
@@ -316,10 +338,10 @@ __device__ __forceinline__ void flow_early(EarlyScalars& q, int G, int k, bool l
   q.inv_g = 1.0 / q.g;
   if ((threadIdx.x & 31) == 0) sh.sc[5] = q.rr;
 }
-// Leaves alpha in sh.ea[k & 1] and the stop status in sh.isc[0].
-__device__ __forceinline__ void flow_late(EarlyScalars& q, int G, int k, Shared& sh) {
+// Leaves alpha in fs.ea[k & 1] and the stop status in sh.isc[0].
+__device__ __forceinline__ void flow_late(EarlyScalars& q, int G, int k, Flow64Shared& fs, Shared& sh) {
   const int lane = threadIdx.x & 31;
-  const double dl = flow_total(2, G, sh);
+  const double dl = flow_total(2, G, fs);
   const double den = k > 0 ? fma(q.m, q.inv_ga, dl) : dl;
   double alpha;
   int st = q.st;
@@ -335,7 +357,7 @@ __device__ __forceinline__ void flow_late(EarlyScalars& q, int G, int k, Shared&
   if (lane == 0) {
     if (st < 0 && !(positive_bits(q.g) && positive_bits(alpha) && finite_bits(alpha))) st = CGP_ERR_BREAKDOWN;
     sh.isc[0] = st;
-    sh.ea[k & 1] = alpha;
+    fs.ea[k & 1] = alpha;
   }
   q.den = den;
 }
@@ -382,11 +404,12 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
   double* const R0 = d.pub64 + 4 * n;                // r of a pass's start, for the ghost rows
   int* const mark = reinterpret_cast<int*>(d.z);     // rows that another block reads
 
-  // shared memory: own vectors, the product's input (CSR: own rows and halo;
+  // shared memory: this form's state, own vectors, the product's input (CSR: own rows and halo;
   // stencil: the padded box), D^-1 and ghost r, s, w of the halo, the system,
   // its indices, and one byte per own row (published or not)
   const bool st = d.stencil;
-  double* base = reinterpret_cast<double*>(dsm);
+  Flow64Shared& fs = *reinterpret_cast<Flow64Shared*>(dsm);
+  double* base = reinterpret_cast<double*>(dsm + sizeof(Flow64Shared));
   double* x = base;
   double* r = base + chunk;
   double* ua = base + 2 * chunk;     // u_k and u_(k+1) alternate
@@ -486,7 +509,7 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
     return;
   }
   const double stop = d.tol * bnorm, stop2 = stop * stop;
-  if (tid < 2) signal_init(&sh.sig[tid]);   // the barriers of the next passes order that before any use
+  if (tid < 2) signal_init(&fs.sig[tid]);   // the barriers of the next passes order that before any use
   if (tid == 0) sh.sc[4] = stop2;   // the test ||r||^2 <= (tol ||b||)^2 needs no square root
 
   int its = 0, restarts = 0, status = CGP_ERR_NOT_CONVERGED, pending = -1;
@@ -535,8 +558,8 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
         g = fma(ri, ui, g);
         rr = fma(ri, ri, rr);
       }
-      sh.ev[0][tid] = g;
-      sh.ev[1][tid] = rr;
+      fs.ev[0][tid] = g;
+      fs.ev[1][tid] = rr;
     }
     if (tid == 0) sh.tflag = 1;
     int k = 0;                           // products formed in this pass, less one
@@ -561,11 +584,11 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
         named_sync(2, ct);
         if (warp == 0) {
           flow_block_sum(2, act, flow_line(d, 1, red, lb), red, sh);
-          if (tid == 0) signal_give(&sh.sig[1]);
+          if (tid == 0) signal_give(&fs.sig[1]);
         }
         // ---- p_(k-1) = u_(k-1) + beta p_(k-2), x += alpha p_(k-1) while the word travels ----
         if (k > 0) {
-          const double alpha = sh.ea[(k - 1) & 1], beta = sh.eb[(k - 1) & 1];
+          const double alpha = fs.ea[(k - 1) & 1], beta = fs.eb[(k - 1) & 1];
           for (int i = tid; i < nloc; i += ct) {
             const double pi = k == 1 ? up[i] : fma(beta, p[i], up[i]);
             p[i] = pi;
@@ -573,15 +596,15 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
           }
         }
         // ---- s_k = w_k + beta_k s_(k-1), once beta_k is known ----
-        if (!signal_wait(&sh.sig[0], phase, d)) sh.tflag = 0;
-        const double beta = sh.eb[k & 1];
+        if (!signal_wait(&fs.sig[0], phase, d)) sh.tflag = 0;
+        const double beta = fs.eb[k & 1];
         for (int i = tid; i < nloc; i += ct) s[i] = k == 0 ? w[i] : fma(beta, s[i], w[i]);
       } else {
         const int nt = bd - ct, cw = warp - ow;
         // ---- the early words: (r,u) and (r,r) ----
         if (cw < act) {
-          flow_warp_sum(sh.ev[0][tid - ct], 0, cw, sh);
-          flow_warp_sum(sh.ev[1][tid - ct], 1, cw, sh);
+          flow_warp_sum(fs.ev[0][tid - ct], 0, cw, sh);
+          flow_warp_sum(fs.ev[1][tid - ct], 1, cw, sh);
         }
         named_sync(3, nt);
         if (warp >= nw - 2) {   // two warps that do not poll
@@ -590,19 +613,19 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
         }
         if (cw < G) {
           ulonglong2 late = make_ulonglong2(0ull, 0ull);
-          if (!flow_poll<2>(d, 0, red, cw, G, 0, late, sh)) sh.tflag = 0;
+          if (!flow_poll<2>(d, 0, red, cw, G, 0, late, fs)) sh.tflag = 0;
           named_sync(1, 32 * (G + 1));
-          if (patient && !signal_wait(&sh.sig[1], phase, d)) sh.tflag = 0;
-          if (!flow_poll<1>(d, 1, red, cw, G, 2, late, sh)) sh.tflag = 0;
+          if (patient && !signal_wait(&fs.sig[1], phase, d)) sh.tflag = 0;
+          if (!flow_poll<1>(d, 1, red, cw, G, 2, late, fs)) sh.tflag = 0;
           named_sync(1, 32 * (G + 1));
         } else if (cw == G) {
           named_sync(1, 32 * (G + 1));
-          flow_early(es, G, k, its + k >= d.max_it, sh);
+          flow_early(es, G, k, its + k >= d.max_it, fs, sh);
           named_sync(1, 32 * (G + 1));
-          flow_late(es, G, k, sh);
+          flow_late(es, G, k, fs, sh);
         } else {
           // ---- the halo's w: other blocks store theirs about when this one does ----
-          if (patient && !signal_wait(&sh.sig[1], phase, d)) sh.tflag = 0;
+          if (patient && !signal_wait(&fs.sig[1], phase, d)) sh.tflag = 0;
           PollLimit lim(d);
           constexpr int B = 4;   // loads of a thread in flight
           const int ht = nt - 32 * (G + 1);
@@ -629,7 +652,7 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
         if (stop_st != CGP_OK) pending = stop_st;
         break;
       }
-      const double alpha = sh.ea[k & 1], beta = sh.eb[k & 1];
+      const double alpha = fs.ea[k & 1], beta = fs.eb[k & 1];
       if (tid < ct) {
         // ---- own rows: r, u_(k+1) and their dot products ----
         double g = 0.0, rr = 0.0;
@@ -642,8 +665,8 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
           g = fma(ri, ui, g);
           rr = fma(ri, ri, rr);
         }
-        sh.ev[0][tid] = g;
-        sh.ev[1][tid] = rr;
+        fs.ev[0][tid] = g;
+        fs.ev[1][tid] = rr;
       } else {
         // ---- ghost rows: s, r, u_(k+1) ----
         for (int h = bd - 1 - tid; h < nh; h += bd - ct) {
@@ -709,9 +732,9 @@ __device__ __forceinline__ void flow_put_f(const Desc& d, int lb, int red, int a
 }
 
 // Warp q < G: wait for the words of the blocks 32 q + lane (+ 32 G ...); the
-// warp's share of the totals goes to sh.pf[c][q] (fixed order: the same bits
+// warp's share of the totals goes to fs.pf[c][q] (fixed order: the same bits
 // in every block).
-__device__ __forceinline__ bool flow_poll_f(const Desc& d, int red, int q, int G, Shared& sh) {
+__device__ __forceinline__ bool flow_poll_f(const Desc& d, int red, int q, int G, Flow32Shared& fs) {
   const int lane = threadIdx.x & 31;
   PollLimit lim(d);
   const unsigned tag = (unsigned)(red + 1);
@@ -733,7 +756,7 @@ __device__ __forceinline__ bool flow_poll_f(const Desc& d, int red, int q, int G
   }
 #pragma unroll
   for (int c = 0; c < 3; ++c) acc[c] = warp_sum(acc[c]);
-  if (lane < 3) sh.pf[lane][q] = lane == 0 ? acc[0] : (lane == 1 ? acc[1] : acc[2]);
+  if (lane < 3) fs.pf[lane][q] = lane == 0 ? acc[0] : (lane == 1 ? acc[1] : acc[2]);
   return true;
 }
 
@@ -743,9 +766,10 @@ __device__ __forceinline__ bool finite_bits(float x) { return ((__float_as_uint(
 // alpha and beta, fsc[3] ||r_0||^2 of the sweep, fsc[4] and fsc[5] the stop
 // bounds, isc[0] the stop flag (0: stop, 1: non-finite, 2: breakdown); gamma
 // and alpha of the last iteration stay with the warp in old[].
-__device__ __forceinline__ void flow_scalars_f(int G, int k, bool last, float (&old)[2], Shared& sh) {
+__device__ __forceinline__ void flow_scalars_f(int G, int k, bool last, float (&old)[2], Flow32Shared& fs,
+                                                Shared& sh) {
   const int lane = threadIdx.x & 31, c = lane >> 3, q = lane & 7;
-  float v = c < 3 && q < G ? sh.pf[c][q] : 0.0f;
+  float v = c < 3 && q < G ? fs.pf[c][q] : 0.0f;
 #pragma unroll
   for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   const float g = __shfl_sync(0xffffffffu, v, 0), dl = __shfl_sync(0xffffffffu, v, 8);
@@ -766,8 +790,8 @@ __device__ __forceinline__ void flow_scalars_f(int G, int k, bool last, float (&
   if (lane == 0) {
     if (k == 0) sh.fsc[3] = rr;
     sh.isc[0] = st;
-    sh.abf[k & 1][0] = alpha;
-    sh.abf[k & 1][1] = beta;
+    fs.abf[k & 1][0] = alpha;
+    fs.abf[k & 1][1] = beta;
   }
   old[0] = g;
   old[1] = alpha;
@@ -809,7 +833,8 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
   float* const R0 = d.f32pub + 4 * n;                // r of a sweep's start, for the ghost rows
   int* const mark = reinterpret_cast<int*>(d.z);     // rows that another block reads
 
-  float* f = reinterpret_cast<float*>(dsm);
+  Flow32Shared& fs = *reinterpret_cast<Flow32Shared*>(dsm);
+  float* f = reinterpret_cast<float*>(dsm + sizeof(Flow32Shared));
   float* ir = f;
   float* iu = f + chunk;
   float* iw = f + 2 * chunk;
@@ -1043,7 +1068,7 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
       flow_put_f(d, lb, red, act, v3, sh);
       // ---- p_(k-1) = u_(k-1) + beta p_(k-2), e += alpha p_(k-1), while the words travel ----
       if (k > 0) {
-        const float alpha = sh.abf[(k - 1) & 1][0], beta = sh.abf[(k - 1) & 1][1];
+        const float alpha = fs.abf[(k - 1) & 1][0], beta = fs.abf[(k - 1) & 1][1];
         own_rows([&](int q, int i) {
           const float uo = VREG ? vq[q] : iu[i];
           const float pi = k == 1 ? uo : fmaf(beta, ip[i], uo);
@@ -1070,9 +1095,9 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
           }
         }
       }
-      if (warp < G && !flow_poll_f(d, red, warp, G, sh)) sh.tflag = 0;
+      if (warp < G && !flow_poll_f(d, red, warp, G, fs)) sh.tflag = 0;
       __syncthreads();
-      if (warp == 0) flow_scalars_f(G, k, total + k >= d.max_it, old, sh);
+      if (warp == 0) flow_scalars_f(G, k, total + k >= d.max_it, old, fs, sh);
       __syncthreads();
       if (!sh.tflag) return;
       ++red;
@@ -1081,7 +1106,7 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
         bad = st == 1;
         break;
       }
-      const float alpha = sh.abf[k & 1][0], beta = sh.abf[k & 1][1];
+      const float alpha = fs.abf[k & 1][0], beta = fs.abf[k & 1][1];
       // ---- own rows and ghost rows: s, r, u_(k+1) ----
       own_rows([&](int q, int i) {
         const float wi = R > 0 ? wq[q] : iw[i];
@@ -1133,14 +1158,14 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
 }
 
 // The solve loop of a system in the general kernels: dataflow iterations where
-// its rows are resident, its reductions tagged and its blocks large enough
-// (cgp_flow.cu has kernels of their own for the FP32 register rows), the barrier
-// forms otherwise.
+// the launch asked for them (d.flow: rows resident, reductions tagged, blocks of
+// at least kFlowMinBlock threads; cgp_flow.cu has kernels of their own for the
+// FP32 register rows), the barrier forms otherwise.
 template <int T, bool RES>
 __device__ __forceinline__ void solve_any(const Desc& d, int lb, Shared& sh) {
   if (d.mixed) {
     if constexpr (RES) {
-      if (d.tagged && blockDim.x >= kFlowMinBlock) {
+      if (d.flow) {
         solve_mixed_flow<T, 0>(d, lb, sh);
         return;
       }
@@ -1150,7 +1175,7 @@ __device__ __forceinline__ void solve_any(const Desc& d, int lb, Shared& sh) {
     solve_fp64<T, RES>(d, lb, sh);
   } else {
     if constexpr (RES) {
-      if (d.tagged && blockDim.x >= kFlowMinBlock) {
+      if (d.flow) {
         solve_fp64_flow<T>(d, lb, sh);
         return;
       }

@@ -137,6 +137,7 @@ struct LaunchPlan {
   bool res = false;
   bool stencil = false;   // resident O-grid tiles with the stencil product
   bool pl = false;        // ... in the pipelined iteration (solve_fp64_pl)
+  bool flow = false;      // dataflow iterations
   HaloPlan halo;
 };
 
@@ -467,15 +468,6 @@ BatchFn resident_batched_kernel_for(SolverKind& kind, int lanes, int block) {
   return batched_kernel_for(lanes, true);
 }
 
-// The mixed kernel with register rows (cgp_flow.cu) in place of `fn` where it
-// applies: tagged reductions, one lane per row, and no more rows a thread than
-// it holds.
-const void* flow_or(const void* fn, SolverKind kind, int lanes, int flags, int chunk, int block, bool batched) {
-  if (lanes != 1 || !(flags & 8) || kind != KIND_MIXED) return fn;
-  const void* f = mixed_flow_kernel_ptr(chunk, block, batched);
-  return f ? f : fn;
-}
-
 // Dynamic shared memory of a block that keeps its rows resident: the classic
 // FP64 solver needs seven vectors, the halo buffer and an FP64 CSR slice; the
 // single-reduction FP64 solver nine vectors, the halo buffer, D^-1 of the
@@ -495,7 +487,6 @@ size_t res_smem_bytes(SolverKind kind, int chunk, const HaloPlan& hp) {
     s = 8 * ((size_t)12 * chunk + 5 * (size_t)hp.max_halo + hp.max_nnz) + ints;
   else
     s = 8 * ((size_t)10 * chunk + 5 * (size_t)hp.max_halo + hp.max_nnz) + ints;
-  s += chunk;   // dataflow iterations: which rows other blocks read
   return (s + 15) / 16 * 16;
 }
 
@@ -509,11 +500,11 @@ size_t res_smem_rows(SolverKind kind, int chunk, int nnz) {
 
 // Dynamic shared memory of a resident single-reduction FP64 block on O-grid
 // tiles: nine vectors, the padded box, D^-1 of the halo, seven coefficient
-// planes, ghost r, s, w of the halo; box positions of the rows and the halo,
-// the halo's global rows, and one byte per row.
+// planes, three halo buffers; box positions of the rows and the halo, and the
+// halo's global rows.
 size_t res_smem_stencil(int chunk, int max_halo, int box_cap) {
   const size_t s = 8 * ((size_t)16 * chunk + (size_t)box_cap + 4 * (size_t)max_halo) +
-                   4 * ((size_t)chunk + 2 * (size_t)max_halo) + chunk;
+                   4 * ((size_t)chunk + 2 * (size_t)max_halo);
   return (s + 15) / 16 * 16;
 }
 
@@ -525,6 +516,60 @@ size_t res_smem_stencil_pl(int chunk, int max_halo, int box_cap) {
   const size_t s = 8 * ((size_t)18 * chunk + (size_t)box_cap + (size_t)max_halo) +
                    4 * (2 * (size_t)chunk + 2 * (size_t)max_halo);
   return (s + 15) / 16 * 16;
+}
+
+// Dynamic shared memory that a block of `fn` may ask for.
+size_t smem_limit(const void* fn, int device) {
+  cudaFuncAttributes fa{};
+  if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (size_t)std::max(0, optin_smem(device) - (int)fa.sharedSizeBytes - 1024);
+}
+
+// Kernel of a resident launch and whether it runs dataflow iterations.
+struct ResidentLaunch {
+  const void* fn = nullptr;   // NULL: the rows cannot be resident
+  size_t smem = 0;
+  bool flow = false;
+};
+
+// Resident launch of `blocks` blocks of at most `chunk` rows: `fn`, whose barrier
+// form needs `smem` bytes a block, or the dataflow iterations where they are asked
+// for (tagged reductions, kinds that have them, large enough blocks) and their
+// additional shared memory fits too; a system that only the barrier form can keep
+// resident runs that one.  The mixed solver's register rows (cgp_flow.cu) have
+// kernels of their own.
+ResidentLaunch resident_launch(const void* fn, SolverKind kind, int lanes, int flags, int chunk, int block,
+                               size_t smem, int blocks, int device, bool batched) {
+  ResidentLaunch out;
+  auto fits = [&](const void* f, size_t bytes) {
+    if (bytes > smem_limit(f, device)) return false;
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, block, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return per_sm * dev_info(device).sms >= blocks;
+  };
+  if ((flags & 24) && (kind == KIND_MIXED || kind == KIND_FP64_SR) && block >= kFlowMinBlock) {
+    const void* f = kind == KIND_MIXED && lanes == 1 && (flags & 8) ? mixed_flow_kernel_ptr(chunk, block, batched) : nullptr;
+    const size_t bytes = smem + flow_smem_bytes(kind == KIND_MIXED, chunk);
+    for (const void* g : {f, fn})
+      if (g && fits(g, bytes)) {
+        out.fn = g;
+        out.smem = bytes;
+        out.flow = true;
+        return out;
+      }
+  }
+  if (fits(fn, smem)) {
+    out.fn = fn;
+    out.smem = smem;
+  }
+  return out;
 }
 
 // Bound on the barrier epochs of one solve (the counter must stay below 2^31).
@@ -574,24 +619,14 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
     const int chunk = (n + nblk - 1) / nblk;
     // bit 4 with the tiles: the pipelined iteration, given three polling warps and five computing ones
     const bool pl = (tu.flags & 16) && block >= 256 && nblk <= 2048;
-    PcgFn fnr = pcg_kernel_for(lanes, true);
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, (const void*)fnr) != cudaSuccess) {
-      cudaGetLastError();
-      return CGP_OK;
-    }
-    const size_t limit = (size_t)std::max(0, optin_smem(device) - (int)fa.sharedSizeBytes - 1024);
     const size_t smem = pl ? res_smem_stencil_pl(chunk, ps->st_max_halo, ps->box_cap)
                            : res_smem_stencil(chunk, ps->st_max_halo, ps->box_cap);
-    if (smem > limit) return CGP_OK;
-    if (cudaFuncSetAttribute((const void*)fnr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return CGP_OK;
-    }
-    if (coresident_blocks(fnr, block, device, smem) < nblk) return CGP_OK;
-    out.fn = fnr;
-    out.smem = smem;
+    const ResidentLaunch rl = resident_launch(pcg_kernel_for(lanes, true), pl ? KIND_FP64_PIPE : KIND_FP64_SR,
+                                              lanes, tu.flags, chunk, block, smem, nblk, device, false);
+    if (!rl.fn) return CGP_OK;
+    out.fn = rl.fn;
+    out.smem = rl.smem;
+    out.flow = rl.flow;
     out.halo_cap = ps->st_max_halo;
     out.res = true;
     out.stencil = true;
@@ -604,14 +639,7 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
   const int rough_nnz = hrp[std::min(n, chunk)] - hrp[0];
   SolverKind kind = solver_kind(mixed, tu.flags);
   PcgFn fnr = resident_kernel_for(kind, lanes, block);
-  fnr = flow_or(fnr, kind, lanes, tu.flags, chunk, block, false);
-  cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, (const void*)fnr) != cudaSuccess) {
-    cudaGetLastError();
-    return CGP_OK;
-  }
-  const size_t limit = (size_t)std::max(0, optin_smem(device) - (int)fa.sharedSizeBytes - 1024);
-  if (res_smem_rows(kind, chunk, rough_nnz) > limit) return CGP_OK;
+  if (res_smem_rows(kind, chunk, rough_nnz) > smem_limit(fnr, device)) return CGP_OK;
   HaloPlan hp;
   if (ps) {
     hp = ps->plan;
@@ -619,31 +647,17 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
     int st = get_halo_plan(m, nblk, hp);
     if (st != CGP_OK) return st;
   }
-  const size_t smem = res_smem_bytes(kind, chunk, hp);
-  if (smem > limit) return CGP_OK;
-  if (cudaFuncSetAttribute((const void*)fnr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return CGP_OK;
-  }
-  if (coresident_blocks(fnr, block, device, smem) < nblk) return CGP_OK;
-  out.fn = fnr;
-  out.smem = smem;
+  const ResidentLaunch rl = resident_launch(fnr, kind, lanes, tu.flags, chunk, block,
+                                            res_smem_bytes(kind, chunk, hp), nblk, device, false);
+  if (!rl.fn) return CGP_OK;
+  out.fn = rl.fn;
+  out.smem = rl.smem;
+  out.flow = rl.flow;
   out.nnz_cap = hp.max_nnz;
   out.halo_cap = hp.max_halo;
   out.res = true;
   out.halo = hp;
   return CGP_OK;
-}
-
-// Dynamic shared memory that a block of `fn` may ask for.
-size_t smem_limit(const void* fn, int device) {
-  cudaFuncAttributes fa{};
-  if (cudaFuncGetAttributes(&fa, fn) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return (size_t)std::max(0, optin_smem(device) - (int)fa.sharedSizeBytes - 1024);
 }
 
 // Whether the rows of a renumbered FP64 launch can be resident at all: what its
@@ -656,7 +670,7 @@ bool renumbered_rows_can_fit(const cgp_mesh_impl* m, int nblk, int block, bool t
   SolverKind kind = KIND_FP64_SR;
   const PcgFn fn = resident_kernel_for(kind, 1, block);
   const size_t need = tiles ? res_smem_stencil(chunk, 0, chunk) : res_smem_rows(kind, chunk, nnz);
-  return need <= smem_limit((const void*)fn, m->device);
+  return need <= smem_limit(fn, m->device);
 }
 
 void free_perm_system(PermSystem& ps) {
@@ -779,6 +793,7 @@ Desc make_desc(cgp_mesh_impl* m, const double* b, double* x, const cgp_solve_opt
   d.mixed = o.precision == CGP_MIXED ? 1 : 0;
   d.classic = (flags & 2) ? 1 : 0;
   d.pipelined = (flags & 16) ? 1 : 0;
+  d.flow = plan.flow ? 1 : 0;
   d.tagged = (flags & 24) ? 1 : 0;   // the pipelined iteration reads its reductions from tagged slots
   d.res_nnz_cap = plan.nnz_cap;
   d.halo_cap = plan.halo_cap;
@@ -1068,13 +1083,7 @@ int batch_plan(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts& o) {
   BatchFn fnr = resident_batched_kernel_for(kind, lanes, block);
   int max_chunk = 1;
   for (int i = 0; i < count; ++i) max_chunk = std::max(max_chunk, (B->meshes[i]->n_c + nb[i] - 1) / nb[i]);
-  fnr = flow_or(fnr, kind, lanes, sh.flags, max_chunk, block, true);
-  cudaFuncAttributes fa{};
-  if (res && cudaFuncGetAttributes(&fa, (const void*)fnr) != cudaSuccess) {
-    cudaGetLastError();
-    res = false;
-  }
-  const size_t limit = res ? (size_t)std::max(0, optin_smem(B->device) - (int)fa.sharedSizeBytes - 1024) : 0;
+  const size_t limit = res ? smem_limit(fnr, B->device) : 0;
   for (int i = 0; res && i < count; ++i) {
     cgp_mesh_impl* m = B->meshes[i];
     const int chunk = (m->n_c + nb[i] - 1) / nb[i];
@@ -1088,21 +1097,11 @@ int batch_plan(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts& o) {
     smem = std::max(smem, res_smem_bytes(kind, chunk, hp[i]));
     if (smem > limit) res = false;
   }
-  if (res) {
-    if (cudaFuncSetAttribute((const void*)fnr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      res = false;
-    } else {
-      int per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fnr, block, smem) != cudaSuccess) {
-        cudaGetLastError();
-        per_sm = 0;
-      }
-      if (per_sm * sms < total) res = false;
-    }
-  }
-  if (!res) smem = 0;
+  ResidentLaunch rl;
+  if (res) rl = resident_launch(fnr, kind, lanes, sh.flags, max_chunk, block, smem, total, B->device, true);
+  res = rl.fn != nullptr;
+  fnr = rl.fn;
+  smem = rl.smem;
   B->waves.assign(1, cgp_batch_s::Wave{total, 0, res, smem, res ? fnr : fn0});
   // descriptors
   std::vector<Desc> desc(count);
@@ -1115,6 +1114,7 @@ int batch_plan(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts& o) {
     lp.block = block;
     if (res) {
       lp.res = true;
+      lp.flow = rl.flow;
       lp.nnz_cap = hp[i].max_nnz;
       lp.halo_cap = hp[i].max_halo;
       lp.halo = hp[i];
@@ -1169,10 +1169,8 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
   const int count = B->count;
   SolverKind kind = solver_kind(mixed, sh.flags);
   BatchFn fnr = resident_batched_kernel_for(kind, lanes, block);
-  cudaFuncAttributes fa{};
-  bool can_res = !(sh.flags & 1) && cudaFuncGetAttributes(&fa, (const void*)fnr) == cudaSuccess;
-  if (!can_res) cudaGetLastError();
-  const size_t limit = can_res ? (size_t)std::max(0, optin_smem(B->device) - (int)fa.sharedSizeBytes - 1024) : 0;
+  const size_t limit = (sh.flags & 1) ? 0 : smem_limit(fnr, B->device);
+  const bool can_res = limit > 0;
   const int rows = 256 << ((sh.flags >> 5) & 3);
   std::vector<int> nb(count), order(count);
   for (int i = 0; i < count; ++i) {
@@ -1225,7 +1223,6 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
     size_t smem = 0;
     int max_chunk = 1;
     for (int i : grp) max_chunk = std::max(max_chunk, (B->meshes[i]->n_c + nb[i] - 1) / nb[i]);
-    const BatchFn fnw = flow_or(fnr, kind, lanes, flags, max_chunk, block, true);   // this wave's kernel
     std::vector<HaloPlan> hp(count);
     for (int i : grp) {
       if (!res) break;
@@ -1241,16 +1238,10 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
       smem = std::max(smem, res_smem_bytes(kind, chunk, hp[i]));
       if (smem > limit) res = false;
     }
-    if (res) {
-      int per_sm = 0;
-      if (cudaFuncSetAttribute((const void*)fnw, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)std::max(smem, max_smem)) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fnw, block, smem) != cudaSuccess) {
-        cudaGetLastError();
-        per_sm = 0;
-      }
-      if (per_sm * sms < total) res = false;
-    }
+    ResidentLaunch rl;   // this wave's kernel
+    if (res) rl = resident_launch(fnr, kind, lanes, flags, max_chunk, block, smem, total, B->device, true);
+    res = rl.fn != nullptr;
+    smem = rl.smem;
     if (!res) {
       int per_sm = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)fn0, block, 0) != cudaSuccess) {
@@ -1258,7 +1249,6 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
         return fail(CGP_ERR_CUDA, "batch: occupancy query failed");
       }
       if (per_sm * sms < total) return fail(CGP_ERR_INVALID_ARG, "batch: a wave does not fit the device");
-      smem = 0;
     }
     max_smem = std::max(max_smem, smem);
     const int off = (int)blk_inst.size();
@@ -1270,6 +1260,7 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
       lp.block = block;
       if (res) {
         lp.res = true;
+        lp.flow = rl.flow;
         lp.nnz_cap = hp[i].max_nnz;
         lp.halo_cap = hp[i].max_halo;
         lp.halo = hp[i];
@@ -1282,7 +1273,7 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
       for (int k = 0; k < nb[i]; ++k) blk_inst.push_back(i);
       blk0 += nb[i];
     }
-    waves.push_back(cgp_batch_s::Wave{total, off, res, smem, res ? fnw : fn0});
+    waves.push_back(cgp_batch_s::Wave{total, off, res, smem, res ? rl.fn : fn0});
   }
   if (blk_inst.size() > (size_t)sms * std::max(32, count)) return fail(CGP_ERR_INVALID_ARG, "batch: too many blocks");
   CGP_CUDA(cudaMemcpy(B->d_desc, desc.data(), sizeof(Desc) * count, cudaMemcpyHostToDevice));

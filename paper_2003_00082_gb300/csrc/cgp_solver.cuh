@@ -51,6 +51,7 @@ struct Desc {
   double tol, inner_tol;
   int max_it, max_sweeps, use_x0, mixed;
   int classic;        // FP64: two barriers per iteration (Saad, Alg. 9.1) instead of the single-reduction form
+  int flow;           // rows resident, tagged: dataflow iterations (cgp_flow.cuh)
   int tagged;         // FP64 single-reduction: reductions through tagged slots instead of the group barrier
   int pipelined;      // FP64: pipelined iteration (CSR: kernels of cgp_pipe.cu; tiles: solve_fp64_pl; rows resident only)
   int stencil;        // FP64, rows resident: O-grid tiles with the seven-point stencil product
@@ -107,16 +108,6 @@ struct Shared {
   float fsc[8];
   int flag;
   int tflag;                    // outcome of the last tagged reduction's wait
-  // dataflow iterations: the polling warps' shares of the totals; alpha and beta by iteration
-  // parity; the FP64 rows' parts of (r,u) and (r,r); the signals beta ready
-  // and (w,u) stored
-  long long phi[3][8];
-  int pexp[3][8];
-  float pf[3][8];
-  double ea[2], eb[2];
-  float abf[2][2];
-  double ev[2][MAX_BLOCK / 2];
-  unsigned long long sig[2];
 };
 
 // Barrier over the blocks of one instance (cgp_sync.h): a block that gives
