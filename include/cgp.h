@@ -448,11 +448,14 @@ int cgp_mesh_set_ogrid(cgp_mesh m, int n_theta, int n_r);
  *         bytes); bit 3 (the FP64 single-reduction form, and the FP32 inner
  *         iterations of MIXED) passes each grid-wide reduction through tagged
  *         slots that show by themselves when every block has stored its
- *         partial sum, instead of a read of the slots after a barrier (FP64:
- *         64-bit fixed-point partials, exact up to a truncation 2^-54 below a
- *         warp's or block's largest term); with rows in shared memory and at
- *         least 256 threads per block the iterations then have no grid barrier
- *         at all, the rows other blocks read travelling in tagged words too;
+ *         partial sum, instead of a read of the slots after a barrier; with
+ *         rows in shared memory and at least 256 threads per block (where
+ *         their few KB more than the barrier form's fit) the iterations then
+ *         have no grid barrier at all, the rows other blocks read travelling
+ *         in tagged words too.  FP64 sums there are 128-bit fixed-point ones,
+ *         a block's sent with at least 94 bits below its largest term; with
+ *         the barrier they are 64-bit ones, exact up to a truncation 2^-54
+ *         below a warp's or block's largest term;
  *         bit 4 (FP64, rows in shared memory, at least 256
  *         threads per block and 1, 2 or 4 lanes per row; otherwise the
  *         single-reduction form runs) runs the pipelined iteration of

@@ -132,6 +132,60 @@ CGP_HD inline double to_double(I128 X, int E) {
   return from_bits(sign | ((uint64_t)biased << 52) | (mant & ((1ull << 52) - 1)));
 }
 
+// The same for the usual case, a normal result: the leading 64 bits with the
+// rest as a sticky bit, rounded to 53 by an integer add whose carry runs into the
+// exponent.
+CGP_HD inline double to_double_normal(I128 X, int E) {
+  const bool negative = X < 0;
+  U128 U = negative ? (U128)(-X) : (U128)X;
+  const uint64_t h = (uint64_t)(U >> 64);
+  const int z = h ? clz64(h) : 64 + clz64((uint64_t)U);
+  const int biased = 127 - z + E - 106;
+  if (U == 0 || biased <= 0 || biased >= 2046 || E >= kBadExp) return to_double(X, E);
+  U <<= z;
+  const uint64_t top = (uint64_t)(U >> 64);
+  uint64_t m = top >> 11;
+  const unsigned rest = (unsigned)(top & 0x7FFu) | ((uint64_t)U ? 1u : 0u);
+  m += rest > 0x400u || (rest == 0x400u && (m & 1u)) ? 1u : 0u;
+  return from_bits((negative ? 1ull << 63 : 0ull) + ((uint64_t)(biased - 1) << 52) + m);
+}
+
+// The five 27-bit limbs of a 128-bit integer (the last one signed, 20 bits):
+// limbs of 32 integers add within 32 bits each, and limbs_value puts the sums
+// back together.
+constexpr int kLimbBits = 27, kLimbs = 5;
+CGP_HD inline unsigned limb(I128 X, int i) {
+  const U128 U = (U128)X >> (kLimbBits * i);
+  return i + 1 < kLimbs ? (unsigned)U & ((1u << kLimbBits) - 1) : (unsigned)(int)(X >> (kLimbBits * (kLimbs - 1)));
+}
+CGP_HD inline I128 limbs_value(const unsigned (&s)[kLimbs]) {
+  const uint64_t a = s[0] + ((uint64_t)s[1] << 27), b = s[2] + ((uint64_t)s[3] << 27);   // a + 2^54 b + 2^108 s[4]
+  const uint64_t lo = a + (b << 54);
+  const uint64_t hi = (b >> 10) + ((uint64_t)(int64_t)(int)s[4] << 44) + (lo < a ? 1u : 0u);
+  return (I128)(((U128)hi << 64) | lo);
+}
+
+// One block's partial X (exponent E, |X| < 2^115: at most 256 images) of
+// reduction `red` in one 128-bit word: lo = S[0:64), hi = S[64:104) | E << 40 |
+// tag << 52 with S = X >> kWordShift, so every term keeps at least 94 bits below
+// the block's largest.  A word holds reduction red, an earlier one of the last
+// few, or zeros; the 12-bit tag (its top bit set) tells these apart.
+constexpr int kWordShift = 12;
+CGP_HD inline unsigned word_tag(int red) { return 0x800u | ((unsigned)red & 0x7FFu); }
+CGP_HD inline void pack_word(I128 X, int E, int red, uint64_t& lo, uint64_t& hi) {
+  const I128 S = X >> kWordShift;
+  lo = (uint64_t)S;
+  hi = ((uint64_t)(S >> 64) & 0xFFFFFFFFFFull) | ((uint64_t)(E < kBadExp ? E : 0xFFF) << 40) | ((uint64_t)word_tag(red) << 52);
+}
+CGP_HD inline bool word_current(uint64_t hi, int red) { return (unsigned)(hi >> 52) == word_tag(red); }
+CGP_HD inline int word_exponent(uint64_t hi) {
+  const int e = (int)((hi >> 40) & 0xFFFu);
+  return e == 0xFFF ? kBadExp : e;
+}
+CGP_HD inline I128 word_sum(uint64_t lo, uint64_t hi) {
+  return ((I128)((int64_t)(hi << 24) >> 24) << 64) | (I128)lo;
+}
+
 CGP_HD inline I128 add(I128 a, I128 b) { return a + b; }
 
 // 64-bit images for the tagged reductions of the solver: relative to a

@@ -6,8 +6,8 @@
 // They travel in words that show by themselves whether they are the ones waited
 // for, so a reader polls exactly the data it will use:
 //   - partial sums in tagged 128-bit words (FP64: one per component, {sum,
-//     exponent and reduction number}; FP32: one for all three) on lines that no
-//     other block writes;
+//     exponent, tag}; FP32: one for all three) on lines that no other block
+//     writes;
 //   - w of a row that another block reads, with the reduction's number, in one
 //     128-bit (FP64) or 64-bit (FP32) word.
 // The halo rows' r and s are not published at all: a reader keeps copies of
@@ -49,7 +49,8 @@ constexpr int kMaxShares = 8;   // groups of blocks whose words are folded by on
 // the dynamic part, so that the other forms' blocks stay as small as they are
 // (whole 16-byte units; flow_smem_bytes counts them).
 struct Flow64Shared {
-  long long phi[3][kMaxShares];   // the polling warps' shares of the totals
+  unsigned long long plo[3][kMaxShares];   // the polling warps' shares of the totals
+  long long phi[3][kMaxShares];
   int pexp[3][kMaxShares];
   double ea[2], eb[2];            // alpha and beta by iteration parity
   double ev[2][MAX_BLOCK / 2];    // the rows' parts of (r,u) and (r,r)
@@ -178,46 +179,56 @@ __device__ __forceinline__ void flow_rows(const int* __restrict__ row, const int
 
 // ---- FP64 -------------------------------------------------------------------
 
-// Word of a component: {sum S, exponent E << 48 | reduction + 1}, value
-// S 2^(E - 1074), |S| < 2^62.
-__device__ __forceinline__ void st_sum(void* p, int red, long long S, int E) {
-  st_relaxed_b128(p, (unsigned long long)S, ((unsigned long long)E << 48) | (unsigned)(red + 1));
+// The sums are those of put_partials (cgp_fixed.h): 128-bit integers aligned to
+// the largest exponent, value X 2^(E - 1129).  A block's sum travels in one word
+// (fx::pack_word: 94 bits below its largest term; two words with all of X cost
+// 4300 clocks an iteration on 152 blocks, since polling loads the network), and
+// the fold over the blocks is 128 bits wide again.  A warp's sum is five
+// redux.sync of 27-bit limbs.  Sums of 57-bit images, truncated 2^-54 below the
+// largest term of a warp, block or group, took 7 % less of a solve at 512x256 and
+// 321x163 and 12 % less at 64x32; the 128-bit steps written out on 32-bit words
+// were no faster than the compiler's.
+__device__ __forceinline__ fx::I128 warp_sum_wide(fx::I128 x) {
+  unsigned s[fx::kLimbs];
+#pragma unroll
+  for (int i = 0; i < fx::kLimbs; ++i) s[i] = __reduce_add_sync(0xffffffffu, fx::limb(x, i));
+  return fx::limbs_value(s);
 }
 
-// Exact warp sum of one value per lane, as put_partials64 forms it (each term
-// truncated 2^-54 below the warp's largest), into the block's table.
+// Exact warp sum of one value per lane into the block's table.
 __device__ __forceinline__ void flow_warp_sum(double v, int c, int slot, Shared& sh) {
-  const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx64_exponent(v));
-  const long long S = warp_sum57(E < fx::kBadExp ? fx64_image(v, E) : 0ll);
+  const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx::exponent_of(v));
+  const fx::I128 X = warp_sum_wide(E < fx::kBadExp ? fx::image(v, E) : (fx::I128)0);
   if ((threadIdx.x & 31) == 0) {
-    sh.whi[c][slot] = S;
+    sh.wlo[c][slot] = (unsigned long long)X;
+    sh.whi[c][slot] = (long long)(X >> 64);
     sh.wexp[c][slot] = E;
   }
 }
 // One warp: the block's sum of component c over `act` warps, stored at p.
 __device__ __forceinline__ void flow_block_sum(int c, int act, void* p, int red, Shared& sh) {
   const int lane = threadIdx.x & 31;
-  const long long sw = lane < act ? sh.whi[c][lane] : 0ll;
+  const fx::I128 xw = lane < act ? ((fx::I128)sh.whi[c][lane] << 64) | (fx::I128)sh.wlo[c][lane] : (fx::I128)0;
   const int ew = lane < act ? sh.wexp[c][lane] : 1;
   const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)ew);
-  const long long S = warp_sum57(E < fx::kBadExp ? (sw >> min(E - ew + 5, 63)) : 0ll);
-  if (lane == 0) st_sum(p, red, S, E);
+  const fx::I128 X = warp_sum_wide(E < fx::kBadExp ? fx::sar(xw, E - ew) : (fx::I128)0);
+  uint64_t lo, hi;
+  fx::pack_word(X, E, red, lo, hi);
+  if (lane == 0) st_relaxed_b128(p, lo, hi);
 }
 
 // Polling warp q < G: wait for NC words of kind `kind` of the blocks 32 q + lane
-// (+ 32 G ...); the warp's shares of the totals go to fs.phi/pexp[c0 + c][q],
-// value phi 2^(pexp - 1074), |phi| < 2^62.  A block's partial enters with 57
-// bits relative to the largest one.  The warp that has the early words (kind 0)
-// loads its late word at once, into `late`, so that the load travels while the
-// early words are decoded; the wait for the late words (kind 1) starts from
-// `late`.  False (on every lane) when the wait gave up.
+// (+ 32 G ...); the warp's shares of the totals go to fs.plo/phi/pexp[c0 + c][q].
+// The warp that has the early words (kind 0) loads its late word at once, into
+// `late`, so that the load travels while the early words are decoded; the wait
+// for the late words (kind 1) starts from `late`.  False (on every lane) when the
+// wait gave up.
 template <int NC>
 __device__ __forceinline__ bool flow_poll(const Desc& d, int kind, int red, int q, int G, int c0, ulonglong2& late,
                                           Flow64Shared& fs) {
   const int lane = threadIdx.x & 31;
   PollLimit lim(d);
-  const unsigned tag = (unsigned)(red + 1);
-  long long acc[NC];
+  fx::I128 acc[NC];
   int Ea[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
@@ -238,60 +249,48 @@ __device__ __forceinline__ bool flow_poll(const Desc& d, int kind, int red, int 
       }
       loaded = false;
 #pragma unroll
-      for (int c = 0; c < NC; ++c) have = have && (unsigned)w[c].y == tag;
+      for (int c = 0; c < NC; ++c) have = have && fx::word_current(w[c].y, red);
       if (__all_sync(0xffffffffu, have)) break;
       if (__any_sync(0xffffffffu, lim.expired())) return false;
     }
     if (kind == 0 && base + 32 * G >= d.nblk) late = ld_relaxed_b128(flow_line(d, 1, red, min(32 * q + lane, d.nblk - 1)));
-    int E[NC];
-    long long S[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      const int e = j < d.nblk ? (int)(w[c].y >> 48) : 1;
-      E[c] = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-      S[c] = j < d.nblk && E[c] < fx::kBadExp ? ((long long)w[c].x >> min(E[c] - e + 5, 63)) : 0ll;
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const long long t = warp_sum57(S[c]);
+      const int e = j < d.nblk ? fx::word_exponent(w[c].y) : 1;
+      const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+      const fx::I128 S = fx::sar(fx::word_sum(w[c].x, w[c].y), E - e);
+      const fx::I128 t = warp_sum_wide(j < d.nblk && E < fx::kBadExp ? S : (fx::I128)0);
       if (base == 32 * q) {
         acc[c] = t;
-        Ea[c] = E[c] + 5;
-      } else {   // |acc|, |t| < 2^62: one more bit
-        const int F = max(Ea[c], E[c] + 5);
-        acc[c] = ((acc[c] >> min(F - Ea[c], 63)) + (t >> min(F - (E[c] + 5), 63))) >> 1;
-        Ea[c] = F + 1;
+        Ea[c] = E;
+      } else {
+        const int F = max(Ea[c], E);
+        acc[c] = fx::sar(acc[c], F - Ea[c]) + fx::sar(t, F - E);
+        Ea[c] = F;
       }
     }
   }
   if (lane < NC) {
-    fs.phi[c0 + lane][q] = NC == 2 && lane == 1 ? acc[NC - 1] : acc[0];
+    const fx::I128 a = NC == 2 && lane == 1 ? acc[NC - 1] : acc[0];
+    fs.plo[c0 + lane][q] = (unsigned long long)a;
+    fs.phi[c0 + lane][q] = (long long)(a >> 64);
     fs.pexp[c0 + lane][q] = NC == 2 && lane == 1 ? Ea[NC - 1] : Ea[0];
   }
   return true;
 }
 
-// Nearest double of X 2^(E - 1074), |X| < 2^62: one conversion and an integer
-// add to its exponent where the result is a normal number.
-__device__ __forceinline__ double scaled_double(long long X, int E) {
-  const double y = (double)X;
-  const int e = (int)((fx::dbits(y) >> 52) & 0x7FF) + E - 1074;
-  if (X != 0 && e > 0 && e < 0x7FF) return fx::from_bits(fx::dbits(y) + ((uint64_t)(int64_t)(E - 1074) << 52));
-  return fx::to_double((fx::I128)X, E >= fx::kBadExp ? E : E + kSlot64Shift);   // NaN for a non-finite term
-}
-
 // One warp: the total of component c from its G shares, on every lane.
 __device__ __forceinline__ double flow_total(int c, int G, const Flow64Shared& fs) {
   const int lane = threadIdx.x & 31;
-  const long long x = lane < G ? fs.phi[c][lane] : 0ll;
+  const fx::I128 x = lane < G ? ((fx::I128)fs.phi[c][lane] << 64) | (fx::I128)fs.plo[c][lane] : (fx::I128)0;
   const int e = lane < G ? fs.pexp[c][lane] : 1;
   const int E = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  const long long X = warp_sum57(E < fx::kBadExp ? (x >> min(E - e + 3, 63)) : 0ll);   // eight shares of 59 bits
-  return scaled_double(X, E + 3);
+  return fx::to_double_normal(warp_sum_wide(E < fx::kBadExp ? fx::sar(x, E - e) : (fx::I128)0),
+                              E < fx::kBadExp ? E + fx::kWordShift : E);
 }
 
 // A reciprocal of a normal a to about 22 bits, its exponent set by integer
-// operations so that any exponent moderate() accepts is safe.
+// operations.
 __device__ __forceinline__ double reciprocal_seed(double a) {
   const unsigned long long b = fx::dbits(a);
   const float m = __uint_as_float(0x3F800000u | (unsigned)((b >> 29) & 0x7FFFFFull));   // [1, 2)
@@ -301,9 +300,11 @@ __device__ __forceinline__ double reciprocal_seed(double a) {
   const int e = (int)(f >> 23) - 127 + 2046 - (int)((b >> 52) & 0x7FF);
   return fx::from_bits(((unsigned long long)e << 52) | ((unsigned long long)(f & 0x7FFFFFu) << 29));
 }
-__device__ __forceinline__ bool moderate(double a) {   // a positive normal with room to spare on both sides
+// Positive and within 2^-500 .. 2^500: the quotient of two such numbers and the
+// remainders of flow_late are normal.
+__device__ __forceinline__ bool moderate(double a) {
   const int e = __double2hiint(a) >> 20;
-  return e > 64 && e < 1982;
+  return e > 523 && e < 1523;
 }
 
 // The scalars of an iteration, by one warp:
@@ -311,14 +312,16 @@ __device__ __forceinline__ bool moderate(double a) {   // a positive normal with
 // An FP64 operation takes 64 clocks from issue to use whatever the number of
 // active lanes, and the compiler's division about nine of them in a chain (564
 // clocks).  What depends on gamma and (r,r) alone is done while the product runs
-// (flow_early); after delta one operation gives the denominator, and the
-// quotient takes three more: lane 0 forms it by one residual correction
-// (Markstein's) with the reciprocal that lane 1 refines meanwhile by one Newton
-// step (flow_late).
+// (flow_early), 1 / (gamma alpha) of the iteration before while the early words
+// travel; after delta one operation gives the denominator, and the quotient takes
+// five more: lane 0 corrects it twice by its remainder (Markstein), first with the
+// reciprocal that lane 1 has after one Newton step, then with the one it has after
+// two.  After the first correction the quotient is one unit in the last place off
+// in 1 of 100,000 cases; the second remainder is then exact and the result the
+// correctly rounded quotient, as of a division.
 struct EarlyScalars {
   double g, rr, m;         // gamma, (r,r), -gamma^2
   double inv_g, inv_ga;    // 1 / gamma and, of the iteration before, 1 / (gamma alpha)
-  double den;              // denominator of alpha
   int st;                  // stop status so far (-1: go on)
 };
 // Leaves beta in fs.eb[k & 1] and gives sig[0] once it is there.
@@ -347,9 +350,13 @@ __device__ __forceinline__ void flow_late(EarlyScalars& q, int G, int k, Flow64S
   int st = q.st;
   if (moderate(den) && moderate(q.g)) {
     const double y0 = reciprocal_seed(den);
-    const double t1 = fma(lane == 0 ? q.g : -den, y0, lane == 0 ? 0.0 : 1.0);                   // q0; 1 - den y0
-    const double t2 = fma(lane == 0 ? -den : t1, lane == 0 ? t1 : y0, lane == 0 ? q.g : y0);    // g - den q0; y1
-    alpha = fma(t2, __shfl_sync(0xffffffffu, t2, 1), t1);                                       // lane 0: q0 + rem y1
+    const bool quo = lane == 0;
+    const double t1 = fma(quo ? q.g : -den, y0, quo ? 0.0 : 1.0);              // q0; 1 - den y0
+    const double t2 = fma(quo ? -den : t1, quo ? t1 : y0, quo ? q.g : y0);     // g - den q0; y1
+    const double y1 = __shfl_sync(0xffffffffu, t2, 1);
+    const double t3 = fma(quo ? t2 : -den, y1, quo ? t1 : 1.0);                // q1; 1 - den y1
+    const double t4 = fma(quo ? -den : t3, quo ? t3 : y1, quo ? q.g : y1);     // g - den q1; y2
+    alpha = fma(t4, __shfl_sync(0xffffffffu, t4, 1), t3);                      // lane 0: q1 + rem y2
   } else {
     if (!finite_bits(dl)) st = CGP_ERR_NONFINITE;
     alpha = q.g / den;
@@ -359,7 +366,6 @@ __device__ __forceinline__ void flow_late(EarlyScalars& q, int G, int k, Flow64S
     sh.isc[0] = st;
     fs.ea[k & 1] = alpha;
   }
-  q.den = den;
 }
 
 // Word of row j's w in the publication of reduction `red`.
@@ -619,6 +625,7 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
           if (!flow_poll<1>(d, 1, red, cw, G, 2, late, fs)) sh.tflag = 0;
           named_sync(1, 32 * (G + 1));
         } else if (cw == G) {
+          if (k > 0) es.inv_ga = es.inv_g * (1.0 / fs.ea[(k - 1) & 1]);
           named_sync(1, 32 * (G + 1));
           flow_early(es, G, k, its + k >= d.max_it, fs, sh);
           named_sync(1, 32 * (G + 1));
@@ -676,7 +683,6 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
           gr[h] = rj;
           ext[halo_at(h)] = dih[h] * rj;
         }
-        if (warp == ow + G) es.inv_ga = es.den * es.inv_g * es.inv_g;   // 1 / (gamma alpha) = den / gamma^2
       }
       ++k;
     }
