@@ -544,10 +544,13 @@ struct ResidentLaunch {
 ResidentLaunch resident_launch(const void* fn, SolverKind kind, int lanes, int flags, int chunk, int block,
                                size_t smem, int blocks, int device, bool batched) {
   ResidentLaunch out;
+  // a kernel's limit is shared by every plan that launches it (batches, captured graphs): it is set to the most a
+  // block may have and never lowered to what one plan needs
   auto fits = [&](const void* f, size_t bytes) {
-    if (bytes > smem_limit(f, device)) return false;
+    const size_t limit = smem_limit(f, device);
+    if (bytes > limit) return false;
     int per_sm = 0;
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess ||
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, block, bytes) != cudaSuccess) {
       cudaGetLastError();
       return false;
