@@ -147,21 +147,27 @@ int build_halo_plan(const std::vector<int>& rp, const std::vector<int>& cl, int 
   const int nnz = rp[n];
   const int chunk = (n + nblk - 1) / nblk;
   std::vector<int> lcol(nnz), hptr(nblk + 1, 0), hidx, h;
+  std::vector<int> at(n, -1);   // local index of the current block's halo columns
   HaloPlan p;
   p.nblk = nblk;
   for (int b = 0; b < nblk; ++b) {
     const int r0 = std::min(n, b * chunk), r1 = std::min(n, r0 + chunk), nloc = r1 - r0;
     const int k0 = rp[r0], k1 = rp[r1];
     h.clear();
-    for (int k = k0; k < k1; ++k)
-      if (cl[k] < r0 || cl[k] >= r1) h.push_back(cl[k]);
-    std::sort(h.begin(), h.end());
-    h.erase(std::unique(h.begin(), h.end()), h.end());
     for (int k = k0; k < k1; ++k) {
       const int j = cl[k];
-      lcol[k] = (j >= r0 && j < r1) ? j - r0
-                                    : nloc + (int)(std::lower_bound(h.begin(), h.end(), j) - h.begin());
+      if ((j < r0 || j >= r1) && at[j] < 0) {
+        at[j] = 0;
+        h.push_back(j);
+      }
     }
+    std::sort(h.begin(), h.end());
+    for (size_t q = 0; q < h.size(); ++q) at[h[q]] = nloc + (int)q;
+    for (int k = k0; k < k1; ++k) {
+      const int j = cl[k];
+      lcol[k] = (j >= r0 && j < r1) ? j - r0 : at[j];
+    }
+    for (int j : h) at[j] = -1;
     hptr[b + 1] = hptr[b] + (int)h.size();
     hidx.insert(hidx.end(), h.begin(), h.end());
     p.max_rows = std::max(p.max_rows, nloc);
@@ -200,26 +206,29 @@ int get_halo_plan(cgp_mesh_impl* m, int nblk, HaloPlan& out) {
   return CGP_OK;
 }
 
-// Recursive coordinate bisection of the nodes idx[lo, hi) into k parts whose
+// Recursive coordinate bisection of the nodes p[lo, hi) into k parts whose
 // sizes follow the solver's chunking (every part `chunk` rows but the last):
 // the left side takes k/2 parts, split along the wider side of the bounding
 // box; ties broken by node index, so the partition is deterministic.
-void rcb(std::vector<int>& idx, int lo, int hi, int k, int chunk, const std::vector<double>& xy) {
+struct Point {
+  double c[2];
+  int node;
+};
+void rcb(std::vector<Point>& p, int lo, int hi, int k, int chunk) {
   if (k <= 1 || hi - lo <= 1) return;
   double x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
   for (int q = lo; q < hi; ++q) {
-    const double x = xy[2 * (size_t)idx[q]], y = xy[2 * (size_t)idx[q] + 1];
-    x0 = std::min(x0, x); x1 = std::max(x1, x); y0 = std::min(y0, y); y1 = std::max(y1, y);
+    x0 = std::min(x0, p[q].c[0]); x1 = std::max(x1, p[q].c[0]);
+    y0 = std::min(y0, p[q].c[1]); y1 = std::max(y1, p[q].c[1]);
   }
   const int axis = (x1 - x0) >= (y1 - y0) ? 0 : 1;
   const int k1 = k / 2;
   const int mid = std::min(hi, lo + k1 * chunk);
-  std::nth_element(idx.begin() + lo, idx.begin() + mid, idx.begin() + hi, [&](int a, int b) {
-    const double va = xy[2 * (size_t)a + axis], vb = xy[2 * (size_t)b + axis];
-    return va < vb || (va == vb && a < b);
+  std::nth_element(p.begin() + lo, p.begin() + mid, p.begin() + hi, [axis](const Point& a, const Point& b) {
+    return a.c[axis] < b.c[axis] || (a.c[axis] == b.c[axis] && a.node < b.node);
   });
-  rcb(idx, lo, mid, k1, chunk, xy);
-  rcb(idx, mid, hi, k - k1, chunk, xy);
+  rcb(p, lo, mid, k1, chunk);
+  rcb(p, mid, hi, k - k1, chunk);
 }
 
 // The system of a solve on nblk blocks in the bisection order (built once per
@@ -231,7 +240,36 @@ void rcb(std::vector<int>& idx, int lo, int hi, int k, int chunk, const std::vec
 // coordinates, so every block owns a near-rectangle of the index grid, and
 // the system also carries what the stencil product needs (tile_stencil).
 int tile_stencil(cgp_mesh_impl* m, PermSystem& ps, const std::vector<int>& perm, const std::vector<int>& inv,
-                 const std::vector<double>& K);
+                 const double* K);
+
+// Values of a renumbered system: entry q is the mesh's entry src[q], row r its row
+// perm[r] (the host builds the pattern only; moving the values through it as well
+// was a third of the time of a first solve's preparation at 512x256).
+__global__ void perm_values_kernel(int n, int nnz, const int* __restrict__ perm, const int* __restrict__ src,
+                                   const double* __restrict__ K, const double* __restrict__ dinv,
+                                   const unsigned char* __restrict__ fixed, double* __restrict__ Ko,
+                                   float* __restrict__ Ko32, double* __restrict__ dino, float* __restrict__ dino32,
+                                   unsigned char* __restrict__ fixedo) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < nnz) {
+    const double k = K[src[q]];
+    Ko[q] = k;
+    Ko32[q] = (float)k;
+  }
+  if (q < n) {
+    const int o = perm[q];
+    const double d = dinv[o];
+    dino[q] = d;
+    dino32[q] = (float)d;
+    if (fixed) fixedo[q] = fixed[o];
+  }
+}
+// Stencil planes of a tiled system: coefficient q is the mesh's entry src[q], or zero (-1).
+__global__ void perm_planes_kernel(int count, const int* __restrict__ src, const double* __restrict__ K,
+                                   double* __restrict__ planes) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < count) planes[q] = src[q] >= 0 ? K[src[q]] : 0.0;
+}
 
 int get_perm_system(cgp_mesh_impl* m, int nblk, PermSystem*& out, int tiles = 0) {
   const int dir = m->far_dirichlet;
@@ -242,28 +280,22 @@ int get_perm_system(cgp_mesh_impl* m, int nblk, PermSystem*& out, int tiles = 0)
       return CGP_OK;
     }
   const int n = m->n_c, nnz = m->nnz, chunk = (n + nblk - 1) / nblk;
-  std::vector<double> xy(2 * (size_t)n), K(nnz), dv(n);
-  CGP_CUDA(cudaDeviceSynchronize());
-  CGP_CUDA(cudaMemcpy(xy.data(), m->xy_c, xy.size() * 8, cudaMemcpyDeviceToHost));
-  if (tiles)
-    for (int i = 0; i < n; ++i) {   // (angle index, ring index)
-      xy[2 * (size_t)i] = (double)(i % m->st_nt);
-      xy[2 * (size_t)i + 1] = (double)(i / m->st_nt);
-    }
-  CGP_CUDA(cudaMemcpy(K.data(), dir ? m->Kd : m->K, (size_t)nnz * 8, cudaMemcpyDeviceToHost));
-  CGP_CUDA(cudaMemcpy(dv.data(), dir ? m->dinvd : m->dinv, (size_t)n * 8, cudaMemcpyDeviceToHost));
-  std::vector<unsigned char> fix;
-  if (dir) {
-    fix.resize(n);
-    CGP_CUDA(cudaMemcpy(fix.data(), m->fixed, n, cudaMemcpyDeviceToHost));
+  const double* const K = dir ? m->Kd : m->K;
+  std::vector<Point> pts(n);
+  if (tiles) {
+    for (int j = 0, i = 0; i < n; ++j)   // (angle index, ring index)
+      for (int t = 0; t < m->st_nt; ++t, ++i) pts[i] = Point{{(double)t, (double)j}, i};
+  } else {
+    std::vector<double> xy(2 * (size_t)n);
+    CGP_CUDA(cudaMemcpy(xy.data(), m->xy_c, xy.size() * 8, cudaMemcpyDeviceToHost));
+    for (int i = 0; i < n; ++i) pts[i] = Point{{xy[2 * (size_t)i], xy[2 * (size_t)i + 1]}, i};
   }
-  std::vector<int> perm(n), inv(n);
-  for (int i = 0; i < n; ++i) perm[i] = i;
-  rcb(perm, 0, n, nblk, chunk, xy);
-  for (int b = 0; b < nblk; ++b) {   // mesh order inside every chunk (locality of the slices)
-    const int r0 = std::min(n, b * chunk), r1 = std::min(n, r0 + chunk);
-    std::sort(perm.begin() + r0, perm.begin() + r1);
-  }
+  rcb(pts, 0, n, nblk, chunk);
+  // mesh order inside every chunk (locality of the slices)
+  std::vector<int> perm(n), inv(n), part(n), next(nblk);
+  for (int r = 0; r < n; ++r) part[pts[r].node] = r / chunk;
+  for (int b = 0; b < nblk; ++b) next[b] = std::min(n, b * chunk);
+  for (int i = 0; i < n; ++i) perm[next[part[i]]++] = i;
   for (int i = 0; i < n; ++i) inv[perm[i]] = i;
   PermSystem ps;
   ps.nblk = nblk;
@@ -272,27 +304,23 @@ int get_perm_system(cgp_mesh_impl* m, int nblk, PermSystem*& out, int tiles = 0)
   ps.n = n;
   ps.h_rowptr.assign(n + 1, 0);
   ps.h_col.resize(nnz);
-  std::vector<double> pk(nnz), pd(n);
-  std::vector<float> pk32(nnz), pd32(n);
-  std::vector<unsigned char> pfix(dir ? n : 0);
-  std::vector<std::pair<int, double>> row;
+  std::vector<int> src(nnz);   // the mesh's entry of every entry
   for (int r = 0; r < n; ++r) {
-    const int o = perm[r];
-    row.clear();
-    for (int k = m->h_rowptr[o]; k < m->h_rowptr[o + 1]; ++k) row.push_back({inv[m->h_col[k]], K[k]});
-    std::sort(row.begin(), row.end());
-    const int k0 = ps.h_rowptr[r];
-    for (size_t q = 0; q < row.size(); ++q) {
-      ps.h_col[k0 + q] = row[q].first;
-      pk[k0 + q] = row[q].second;
-      pk32[k0 + q] = (float)row[q].second;
+    const int o = perm[r], k0 = ps.h_rowptr[r];
+    int k1 = k0;
+    for (int k = m->h_rowptr[o]; k < m->h_rowptr[o + 1]; ++k, ++k1) {   // few entries a row: insertion sort
+      const int c = inv[m->h_col[k]];
+      int q = k1;
+      for (; q > k0 && ps.h_col[q - 1] > c; --q) {
+        ps.h_col[q] = ps.h_col[q - 1];
+        src[q] = src[q - 1];
+      }
+      ps.h_col[q] = c;
+      src[q] = k;
     }
-    ps.h_rowptr[r + 1] = k0 + (int)row.size();
-    pd[r] = dv[o];
-    pd32[r] = (float)dv[o];
-    if (dir) pfix[r] = fix[o];
+    ps.h_rowptr[r + 1] = k1;
   }
-  int st = build_halo_plan(ps.h_rowptr, ps.h_col, n, nblk, ps.plan);
+  int st = tiles ? CGP_OK : build_halo_plan(ps.h_rowptr, ps.h_col, n, nblk, ps.plan);   // tiles have halo lists of their own
   if (st != CGP_OK) return st;
   auto al = [](size_t v) { return (v + 255) / 256 * 256; };
   const size_t o_perm = 0, o_rp = o_perm + al((size_t)n * 4), o_col = o_rp + al((size_t)(n + 1) * 4),
@@ -300,7 +328,10 @@ int get_perm_system(cgp_mesh_impl* m, int nblk, PermSystem*& out, int tiles = 0)
                o_d32 = o_d + al((size_t)n * 8), o_b = o_d32 + al((size_t)n * 4), o_x = o_b + al((size_t)n * 8),
                o_f = o_x + al((size_t)n * 8), bytes = o_f + al((size_t)n);
   cudaError_t e = cudaMalloc(&ps.base, bytes);
+  int* d_src = nullptr;
+  if (e == cudaSuccess) e = cudaMalloc(&d_src, (size_t)nnz * 4);
   if (e != cudaSuccess) {
+    cudaFree(ps.base);
     cudaFree(ps.plan.base);
     return cuda_fail(e, "cudaMalloc(permuted system)");
   }
@@ -318,15 +349,19 @@ int get_perm_system(cgp_mesh_impl* m, int nblk, PermSystem*& out, int tiles = 0)
   if (e == cudaSuccess) e = cudaMemcpy(ps.perm, perm.data(), (size_t)n * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(ps.rowptr, ps.h_rowptr.data(), (size_t)(n + 1) * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(ps.col, ps.h_col.data(), (size_t)nnz * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(ps.K, pk.data(), (size_t)nnz * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(ps.K32, pk32.data(), (size_t)nnz * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(ps.dinv, pd.data(), (size_t)n * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(ps.dinv32, pd32.data(), (size_t)n * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && dir) e = cudaMemcpy(ps.fixed, pfix.data(), (size_t)n, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(d_src, src.data(), (size_t)nnz * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    perm_values_kernel<<<(std::max(nnz, n) + 255) / 256, 256>>>(n, nnz, ps.perm, d_src, K, dir ? m->dinvd : m->dinv,
+                                                              dir ? m->fixed : nullptr, ps.K, ps.K32, ps.dinv,
+                                                              ps.dinv32, ps.fixed);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(0);   // the solve runs on a stream of its own
+  cudaFree(d_src);
   if (e != cudaSuccess) {
     cudaFree(ps.base);
     cudaFree(ps.plan.base);
-    return cuda_fail(e, "cudaMemcpy(permuted system)");
+    return cuda_fail(e, "permuted system");
   }
   if (tiles) {
     st = tile_stencil(m, ps, perm, inv, K);
@@ -354,16 +389,25 @@ inline int tile_dj(int k) { return k == 3 || k == 5 ? 1 : (k == 4 || k == 6 ? -1
 // reached across the periodic angle seam is taken through the halo even when
 // the block owns it.
 int tile_stencil(cgp_mesh_impl* m, PermSystem& ps, const std::vector<int>& perm, const std::vector<int>& inv,
-                 const std::vector<double>& K) {
+                 const double* K) {
   const int n = ps.n, nblk = ps.nblk, nt = m->st_nt, chunk = (n + nblk - 1) / nblk;
-  std::vector<double> planes((size_t)kStencil * n, 0.0);
+  std::vector<int> from((size_t)kStencil * n, -1);   // the mesh's entry of every coefficient
+  std::vector<int> ai(n), aj(n);                     // angle and ring of a node
+  for (int j = 0, i = 0; i < n; ++j)
+    for (int t = 0; t < nt; ++t, ++i) {
+      ai[i] = t;
+      aj[i] = j;
+    }
+  int dir_of[9];                                     // stencil entry of (angle, ring) offset
+  std::fill(dir_of, dir_of + 9, -1);
+  for (int q = 0; q < kStencil; ++q) dir_of[3 * (tile_dj(q) + 1) + tile_di(q) + 1] = q;
   std::vector<int> bpos(n), bdim(nblk), hptr(nblk + 1, 0), hidx, hpos;
   int box_cap = 0, max_halo = 0;
   for (int b = 0; b < nblk; ++b) {
     const int r0 = std::min(n, b * chunk), r1 = std::min(n, r0 + chunk);
     int a0 = 1 << 30, a1 = -1, j0 = 1 << 30, j1 = -1;
     for (int r = r0; r < r1; ++r) {
-      const int o = perm[r], i = o % nt, j = o / nt;
+      const int o = perm[r], i = ai[o], j = aj[o];
       a0 = std::min(a0, i); a1 = std::max(a1, i); j0 = std::min(j0, j); j1 = std::max(j1, j);
     }
     const int Ba = r1 > r0 ? a1 - a0 + 3 : 1, Bb = r1 > r0 ? j1 - j0 + 3 : 1;
@@ -371,22 +415,20 @@ int tile_stencil(cgp_mesh_impl* m, PermSystem& ps, const std::vector<int>& perm,
     box_cap = std::max(box_cap, Ba * Bb);
     std::vector<std::pair<int, int>> halo;   // (box position, row)
     for (int r = r0; r < r1; ++r) {
-      const int o = perm[r], i = o % nt, j = o / nt;
+      const int o = perm[r], i = ai[o], j = aj[o];
       bpos[r] = (j - j0 + 1) * Ba + (i - a0 + 1);
     }
     for (int r = r0; r < r1; ++r) {
-      const int o = perm[r], i = o % nt, j = o / nt;
+      const int o = perm[r], i = ai[o], j = aj[o];
       for (int k = m->h_rowptr[o]; k < m->h_rowptr[o + 1]; ++k) {
-        const int c = m->h_col[k], ic = c % nt, jc = c / nt;
-        int di = ic - i;
+        const int c = m->h_col[k];
+        int di = ai[c] - i;
         if (di > 1) di -= nt;
         if (di < -1) di += nt;
-        const int dj = jc - j;
-        int dir = -1;
-        for (int q = 0; q < kStencil; ++q)
-          if (tile_di(q) == di && tile_dj(q) == dj) dir = q;
+        const int dj = aj[c] - j;
+        const int dir = di >= -1 && di <= 1 && dj >= -1 && dj <= 1 ? dir_of[3 * (dj + 1) + di + 1] : -1;
         if (dir < 0) return fail(CGP_ERR_INVALID_ARG, "O-grid tiles: a row's pattern is not the seven-point stencil");
-        planes[(size_t)dir * n + r] = K[k];
+        from[(size_t)dir * n + r] = k;
         const int p = bpos[r] + dj * Ba + di, q = inv[c];
         if (q >= r0 && q < r1 && bpos[q] == p) continue;   // owned, at its own box position
         halo.push_back({p, q});
@@ -410,7 +452,13 @@ int tile_stencil(cgp_mesh_impl* m, PermSystem& ps, const std::vector<int>& perm,
                o_hp = o_bd + al((size_t)nblk * 4), o_hi = o_hp + al((size_t)(nblk + 1) * 4),
                o_hs = o_hi + al(nh * 4), bytes = o_hs + al(nh * 4);
   void* base = nullptr;
-  CGP_CUDA(cudaMalloc(&base, bytes));
+  int* d_from = nullptr;
+  cudaError_t e = cudaMalloc(&base, bytes);
+  if (e == cudaSuccess) e = cudaMalloc(&d_from, from.size() * 4);
+  if (e != cudaSuccess) {
+    cudaFree(base);
+    return cuda_fail(e, "cudaMalloc(O-grid tiles)");
+  }
   char* c = static_cast<char*>(base);
   ps.st_base = base;
   ps.planes = (double*)(c + o_pl);
@@ -421,7 +469,14 @@ int tile_stencil(cgp_mesh_impl* m, PermSystem& ps, const std::vector<int>& perm,
   ps.st_hpos = (int*)(c + o_hs);
   ps.box_cap = box_cap;
   ps.st_max_halo = max_halo;
-  cudaError_t e = cudaMemcpy(ps.planes, planes.data(), planes.size() * 8, cudaMemcpyHostToDevice);
+  e = cudaMemcpy(d_from, from.data(), from.size() * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    const int count = (int)from.size();
+    perm_planes_kernel<<<(count + 255) / 256, 256>>>(count, d_from, K, ps.planes);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+  cudaFree(d_from);
   if (e == cudaSuccess) e = cudaMemcpy(ps.bpos, bpos.data(), (size_t)n * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(ps.bdim, bdim.data(), (size_t)nblk * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(ps.st_hptr, hptr.data(), (size_t)(nblk + 1) * 4, cudaMemcpyHostToDevice);
@@ -430,7 +485,7 @@ int tile_stencil(cgp_mesh_impl* m, PermSystem& ps, const std::vector<int>& perm,
   if (e != cudaSuccess) {
     cudaFree(base);
     ps.st_base = nullptr;
-    return cuda_fail(e, "cudaMemcpy(O-grid tiles)");
+    return cuda_fail(e, "O-grid tiles");
   }
   return CGP_OK;
 }
