@@ -612,7 +612,8 @@ ResidentLaunch resident_launch(const void* fn, SolverKind kind, int lanes, int f
     }
     return per_sm * dev_info(device).sms >= blocks;
   };
-  if ((flags & 24) && (kind == KIND_MIXED || kind == KIND_FP64_SR) && block >= kFlowMinBlock) {
+  if ((flags & 24) && (kind == KIND_MIXED || kind == KIND_FP64_SR) && block >= kFlowMinBlock &&
+      blocks <= kFlowBlocksPerSm * dev_info(device).sms) {
     const void* f = kind == KIND_MIXED && lanes == 1 && (flags & 8) ? mixed_flow_kernel_ptr(chunk, block, batched) : nullptr;
     const size_t bytes = smem + flow_smem_bytes(kind == KIND_MIXED, chunk);
     for (const void* g : {f, fn})
@@ -657,6 +658,7 @@ int plan_solve(cgp_mesh_impl* m, int device, int n, int max_blocks, const Solver
     nblk = std::min(sms, std::max(1, (n + 255) / 256));
   }
   nblk = std::max(1, std::min(nblk, std::min(cap0, n)));
+  if (tu.flags & 24) nblk = std::min(nblk, sms * kTaggedBlocksPerSm);   // lines for the tagged words
   out = LaunchPlan{};
   out.fn = fn0;
   out.nblk = nblk;
@@ -803,10 +805,13 @@ int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps,
 
 }  // namespace
 
+int solver_sms(int device) {
+  const int sms = dev_info(device).sms;
+  return sms > 0 ? sms : 160;
+}
+
 int solver_max_blocks(int device) {
-  int sms = dev_info(device).sms;
-  if (sms <= 0) sms = 160;
-  return sms * 32;  // upper bound on co-resident blocks of >= 64 threads
+  return solver_sms(device) * 32;  // upper bound on co-resident blocks of >= 64 threads
 }
 
 namespace {
@@ -1099,6 +1104,7 @@ int batch_plan(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts& o) {
   }
   int G = per_sm0 * sms;
   if (sh.per_sm > 0) G = std::min(G, sh.per_sm * sms);
+  if (sh.flags & 24) G = std::min(G, sms * kTaggedBlocksPerSm);
   const int count = B->count;
   if (G < count) return fail(CGP_ERR_INVALID_ARG, "batch: more instances than co-resident blocks");
   // blocks per instance in proportion to nnz * sqrt(n) (work of a CG solve on a 2-D mesh)
@@ -1223,7 +1229,8 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
     cudaGetLastError();
     return fail(CGP_ERR_CUDA, "batch: occupancy query failed");
   }
-  const int cap = sms * std::min(std::max(1, sh.per_sm), fit);
+  int cap = sms * std::min(std::max(1, sh.per_sm), fit);
+  if (flags & 24) cap = std::min(cap, sms * kTaggedBlocksPerSm);
   const int count = B->count;
   SolverKind kind = solver_kind(mixed, sh.flags);
   BatchFn fnr = resident_batched_kernel_for(kind, lanes, block);

@@ -41,7 +41,7 @@ struct Desc {
   float* f32own;      // mixed without RES: own r, u, w, p, s, e ([6][n])
   float* fpart;       // mixed: FP32 partial slots [2][NCOMP][part_stride]
   double* part;
-  unsigned long long* tpart;  // tagged slots and records: per block two lines of kLineBytes (banks by parity)
+  unsigned long long* tpart;  // tagged words: lines of kLineBytes, two (banks by parity) or in dataflow form four a block
   unsigned* nflag;    // FP64 pipelined tiles: per block, the count of its published w (release)
   int part_stride;
   unsigned* bar;
@@ -179,7 +179,7 @@ __device__ __forceinline__ unsigned long long* part_slot(const Desc& d, int red,
 // zeroes its slots at the start of a launch.
 __device__ __forceinline__ ulonglong2* tag_slot(const Desc& d, int red, int c, int blk) {
   return reinterpret_cast<ulonglong2*>(reinterpret_cast<unsigned char*>(d.tpart) +
-                                       ((size_t)blk * 4 + (red & 1)) * kLineBytes) + c;
+                                       ((size_t)blk * 2 + (red & 1)) * kLineBytes) + c;
 }
 
 // Sum NC (<= 3) per-thread values over the block; warp c then folds
@@ -1693,7 +1693,7 @@ __device__ void solve_fp64_pl(const Desc& d, int lb, Shared& sh) {
 // block zeroes its words at launch start).  Banks by the reduction's parity.
 __device__ __forceinline__ unsigned long long* ftag_slot(const Desc& d, int red, int c, int blk) {
   return reinterpret_cast<unsigned long long*>(reinterpret_cast<unsigned char*>(d.tpart) +
-                                               ((size_t)blk * 4 + (red & 1)) * kLineBytes) + c;
+                                               ((size_t)blk * 2 + (red & 1)) * kLineBytes) + c;
 }
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
