@@ -524,10 +524,13 @@ int cgp_autotune(cgp_mesh m, int precision, const double* b, double* x, const ch
 int cgp_last_launch(cgp_mesh m, int precision, int* blocks, int* block, int* resident, int* smem_bytes);
 
 /*
- * cgp_barrier_selftest - exercise the persistent solver's grid barrier.
- * Launches nblk co-resident blocks (1 <= nblk <= 1024) of which the last
- * `absent` never arrive; the others give up after spin_ns nanoseconds and the
- * call returns CGP_ERR_TIMEOUT, or CGP_OK when absent == 0.  The GPU context
+ * cgp_barrier_selftest - exercise the persistent solvers' waits.
+ * Launches nblk co-resident blocks (1 <= nblk <= 1024) for each kind of wait
+ * (grid barrier, tagged sums and halo rows of the dataflow iterations in FP64
+ * and FP32, signals inside a block), of which the last `absent` never arrive;
+ * the others give up after spin_ns nanoseconds and the call returns
+ * CGP_ERR_TIMEOUT, or CGP_OK when absent == 0; CGP_ERR_CUDA when a wait ended
+ * that should not have, or a value read through it was wrong.  The GPU context
  * stays usable either way.  Synchronises the stream.
  */
 int cgp_barrier_selftest(int nblk, int absent, long long spin_ns, void* stream);

@@ -373,6 +373,28 @@ __device__ __forceinline__ ulonglong2* flow_w64(const Desc& d, int red, int j) {
   return reinterpret_cast<ulonglong2*>(d.pub64) + (size_t)(red & 1) * d.n + j;
 }
 
+// Thread t of nt: w of the rows hid[0 .. nh) in reduction `red`, as their owners
+// store them.  False when the wait gave up.
+__device__ __forceinline__ bool flow_fetch64(const Desc& d, int red, const int* hid, int nh, double* gw, int t, int nt) {
+  const unsigned long long tag = (unsigned long long)red + 1;
+  PollLimit lim(d);
+  constexpr int B = 4;   // loads of a thread in flight
+  bool ok = true;
+  for (int h = t; h < nh; h += B * nt) {
+    ulonglong2 a[B];
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+      a[q] = h + q * nt < nh ? ld_relaxed_b128(flow_w64(d, red, hid[h + q * nt])) : make_ulonglong2(0ull, tag);
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      while (a[q].y != tag && !lim.expired()) a[q] = ld_relaxed_b128(flow_w64(d, red, hid[h + q * nt]));
+      ok = ok && a[q].y == tag;
+      if (h + q * nt < nh) gw[h + q * nt] = fx::from_bits(a[q].x);
+    }
+  }
+  return ok;
+}
+
 // FP64 Jacobi-PCG in the single-reduction form (solve_fp64_sr describes the
 // recurrences) with rows resident in shared memory and dataflow iterations.
 // The passes around the loop (projections, true residual) use the group
@@ -633,21 +655,7 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
         } else {
           // ---- the halo's w: other blocks store theirs about when this one does ----
           if (patient && !signal_wait(&fs.sig[1], phase, d)) sh.tflag = 0;
-          PollLimit lim(d);
-          constexpr int B = 4;   // loads of a thread in flight
-          const int ht = nt - 32 * (G + 1);
-          for (int h = bd - 1 - tid; h < nh; h += B * ht) {
-            ulonglong2 a[B];
-#pragma unroll
-            for (int q = 0; q < B; ++q)
-              a[q] = h + q * ht < nh ? ld_relaxed_b128(flow_w64(d, red, hid[h + q * ht])) : make_ulonglong2(0ull, tag);
-#pragma unroll
-            for (int q = 0; q < B; ++q) {
-              while (a[q].y != tag && !lim.expired()) a[q] = ld_relaxed_b128(flow_w64(d, red, hid[h + q * ht]));
-              if (a[q].y != tag) sh.tflag = 0;
-              if (h + q * ht < nh) gw[h + q * ht] = fx::from_bits(a[q].x);
-            }
-          }
+          if (!flow_fetch64(d, red, hid, nh, gw, bd - 1 - tid, nt - 32 * (G + 1))) sh.tflag = 0;
         }
       }
       __syncthreads();
@@ -805,6 +813,27 @@ __device__ __forceinline__ void flow_scalars_f(int G, int k, bool last, float (&
 
 __device__ __forceinline__ unsigned long long* flow_w32(const Desc& d, int red, int j) {
   return reinterpret_cast<unsigned long long*>(d.f32pub) + (size_t)(red & 1) * d.n + j;
+}
+
+// As flow_fetch64.
+__device__ __forceinline__ bool flow_fetch32(const Desc& d, int red, const int* hid, int nh, float* gw, int t, int nt) {
+  const unsigned tag = (unsigned)(red + 1);
+  PollLimit lim(d);
+  constexpr int B = 4;   // loads of a thread in flight
+  bool ok = true;
+  for (int h = t; h < nh; h += B * nt) {
+    unsigned long long a[B];
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+      a[q] = h + q * nt < nh ? ld_relaxed_u64(flow_w32(d, red, hid[h + q * nt])) : (unsigned long long)tag << 32;
+#pragma unroll
+    for (int q = 0; q < B; ++q) {
+      while ((unsigned)(a[q] >> 32) != tag && !lim.expired()) a[q] = ld_relaxed_u64(flow_w32(d, red, hid[h + q * nt]));
+      ok = ok && (unsigned)(a[q] >> 32) == tag;
+      if (h + q * nt < nh) gw[h + q * nt] = __uint_as_float((unsigned)a[q]);
+    }
+  }
+  return ok;
 }
 
 // Mixed precision with rows resident: the FP64 refinement and the FP32 inner
@@ -1085,21 +1114,7 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
       }
       // ---- the halo's w, then the sums ----
       if (tid >= f0) {
-        PollLimit lim(d);
-        constexpr int B = 4;   // loads of a thread in flight
-        const int nt = bd - f0;
-        for (int h = tid - f0; h < nh; h += B * nt) {
-          unsigned long long a[B];
-#pragma unroll
-          for (int q = 0; q < B; ++q)
-            a[q] = h + q * nt < nh ? ld_relaxed_u64(flow_w32(d, red, hid[h + q * nt])) : (unsigned long long)tag << 32;
-#pragma unroll
-          for (int q = 0; q < B; ++q) {
-            while ((unsigned)(a[q] >> 32) != tag && !lim.expired()) a[q] = ld_relaxed_u64(flow_w32(d, red, hid[h + q * nt]));
-            if ((unsigned)(a[q] >> 32) != tag) sh.tflag = 0;
-            if (h + q * nt < nh) gw[h + q * nt] = __uint_as_float((unsigned)a[q]);
-          }
-        }
+        if (!flow_fetch32(d, red, hid, nh, gw, tid - f0, bd - f0)) sh.tflag = 0;
       }
       if (warp < G && !flow_poll_f(d, red, warp, G, fs)) sh.tflag = 0;
       __syncthreads();

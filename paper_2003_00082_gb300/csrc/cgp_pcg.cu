@@ -1030,15 +1030,61 @@ int launch_spmv(cgp_mesh_impl* m, int precision, const void* x, void* y, cudaStr
 }
 
 // ---------------------------------------------------------------------------
-// barrier self-test: the last `absent` blocks never arrive
+// self-test of the solvers' grid-wide waits: the last `absent` blocks never
+// arrive.  Kinds: the counter barrier; the words of the FP64 and of the FP32 sums;
+// the words of the FP64 and of the FP32 halo; a signal inside a block (not given
+// when a block is absent).
 // ---------------------------------------------------------------------------
-__global__ void barrier_selftest_kernel(unsigned* bar, int* timeout, int nblk, int absent, long long spin_ns,
-                                        int* ok_count) {
+enum WaitKind { WAIT_BARRIER, WAIT_SUMS64, WAIT_SUMS32, WAIT_HALO64, WAIT_HALO32, WAIT_SIGNAL, WAIT_KINDS };
+constexpr int kSelftestMax = 1024;   // blocks
+
+// Blocks of one warp; d.bar, d.tpart, d.pub64, d.f32pub zeroed, d.n = d.nblk rows, block b owns row b.
+__global__ void wait_selftest_kernel(Desc d, int kind, int absent, int* ok_count) {
   __shared__ Shared sh;
-  if ((int)blockIdx.x >= nblk - absent) return;
-  Group grp{bar, timeout, (unsigned)nblk, 0u, spin_ns};
-  const bool ok = grp.sync(sh);
-  if (threadIdx.x == 0 && ok) atomicAdd(ok_count, 1);
+  __shared__ Flow64Shared f64;
+  __shared__ Flow32Shared f32;
+  __shared__ int rows[kSelftestMax];
+  __shared__ double got[kSelftestMax];
+  const int b = blockIdx.x, lane = threadIdx.x, red = 0;
+  if (b >= d.nblk - absent) return;
+  for (int i = lane; i < d.nblk; i += 32) rows[i] = i;
+  if (lane == 0) signal_init(&f64.sig[0]);
+  __syncthreads();
+  bool ok = false;
+  if (kind == WAIT_BARRIER) {
+    Group grp{d.bar, &d.res->timeout, (unsigned)d.nblk, 0u, d.spin_ns};
+    ok = grp.sync(sh);
+  } else if (kind == WAIT_SUMS64) {
+    uint64_t lo, hi;
+    fx::pack_word((fx::I128)(b + 1) << 60, 1000, red, lo, hi);
+    if (lane < 3) st_relaxed_b128(flow_line(d, lane / 2, red, b) + 16 * (lane % 2), lo, hi);   // two early words, one late
+    ulonglong2 late = make_ulonglong2(0ull, 0ull);
+    ok = flow_poll<2>(d, 0, red, 0, 1, 0, late, f64) && flow_poll<1>(d, 1, red, 0, 1, 2, late, f64);
+    const double one = fx::to_double((fx::I128)1 << 60, 1000), all = 0.5 * d.nblk * (d.nblk + 1);
+    __syncwarp();
+    for (int c = 0; c < 3; ++c) ok = ok && flow_total(c, 1, f64) == all * one;
+  } else if (kind == WAIT_SUMS32) {
+    if (lane == 0)
+      st_relaxed_b128(flow_line(d, 0, red, b), 0ull, ((unsigned long long)(red + 1) << 32) | __float_as_uint(1.0f));
+    ok = flow_poll_f(d, red, 0, 1, f32);
+    __syncwarp();
+    ok = ok && f32.pf[2][0] == (float)d.nblk;
+  } else if (kind == WAIT_HALO64) {
+    if (lane == 0) st_relaxed_b128(flow_w64(d, red, b), fx::dbits(1.0 + b), (unsigned long long)red + 1);
+    ok = flow_fetch64(d, red, rows, d.nblk, got, lane, 32);
+    for (int i = lane; i < d.nblk; i += 32) ok = ok && got[i] == 1.0 + i;
+  } else if (kind == WAIT_HALO32) {
+    if (lane == 0)
+      st_relaxed_u64(flow_w32(d, red, b), ((unsigned long long)(red + 1) << 32) | __float_as_uint(1.0f + b));
+    float* const g = reinterpret_cast<float*>(got);
+    ok = flow_fetch32(d, red, rows, d.nblk, g, lane, 32);
+    for (int i = lane; i < d.nblk; i += 32) ok = ok && g[i] == 1.0f + i;
+  } else {
+    if (lane == 0 && absent == 0) signal_give(&f64.sig[0]);
+    ok = signal_wait(&f64.sig[0], 0u, d);
+  }
+  ok = __all_sync(0xffffffffu, ok);
+  if (lane == 0 && ok) atomicAdd(ok_count, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -1471,34 +1517,52 @@ extern "C" int cgp_last_launch(cgp_mesh m, int precision, int* blocks, int* bloc
 }
 
 extern "C" int cgp_barrier_selftest(int nblk, int absent, long long spin_ns, void* stream) {
-  if (nblk < 1 || nblk > 1024 || absent < 0 || absent >= nblk || spin_ns <= 0)
+  if (nblk < 1 || nblk > kSelftestMax || absent < 0 || absent >= nblk || spin_ns <= 0)
     return fail(CGP_ERR_INVALID_ARG, "cgp_barrier_selftest: need 1 <= nblk <= 1024, 0 <= absent < nblk");
   cudaStream_t s = (cudaStream_t)stream;
   int device = 0;
   CGP_CUDA(cudaGetDevice(&device));
   int per_sm = 0;
-  CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)barrier_selftest_kernel, 64, 0));
+  CGP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)wait_selftest_kernel, 32, 0));
   if (per_sm * dev_info(device).sms < nblk)
     return fail(CGP_ERR_INVALID_ARG, "cgp_barrier_selftest: nblk exceeds the co-resident capacity");
-  void* buf = nullptr;
-  CGP_CUDA(cudaMalloc(&buf, 256));
-  unsigned* bar = (unsigned*)buf;
-  int* timeout = (int*)((char*)buf + 64);
-  int* ok_count = (int*)((char*)buf + 128);
-  int h[2] = {0, 0};
-  cudaError_t e = cudaMemsetAsync(buf, 0, 256, s);
-  if (e == cudaSuccess) {
-    void* args[] = {&bar, &timeout, &nblk, &absent, &spin_ns, &ok_count};
-    e = cudaLaunchCooperativeKernel((const void*)barrier_selftest_kernel, dim3(nblk), dim3(64), args, 0, s);
+  // barrier counter, result record, count of passing blocks; lines; published rows (two banks)
+  const size_t o_res = 256, o_ok = 512, o_line = 768, o_w64 = o_line + (size_t)nblk * 4 * kLineBytes,
+               o_w32 = o_w64 + (size_t)nblk * 32, bytes = o_w32 + (size_t)nblk * 16;
+  static_assert(sizeof(SolveResult) <= 256, "the record fits its slot");
+  char* buf = nullptr;
+  CGP_CUDA(cudaMalloc(&buf, bytes));
+  Desc d{};
+  d.n = d.nblk = nblk;
+  d.bar = (unsigned*)buf;
+  d.res = (SolveResult*)(buf + o_res);
+  d.tpart = (unsigned long long*)(buf + o_line);
+  d.pub64 = (double*)(buf + o_w64);
+  d.f32pub = (float*)(buf + o_w32);
+  d.spin_ns = spin_ns;
+  int* ok_count = (int*)(buf + o_ok);
+  int timed_out = 0, passed = 0, wrong = -1;
+  cudaError_t e = cudaSuccess;
+  for (int kind = 0; kind < WAIT_KINDS && e == cudaSuccess; ++kind) {
+    int h[2] = {0, 0};
+    e = cudaMemsetAsync(buf, 0, bytes, s);
+    if (e == cudaSuccess) {
+      void* args[] = {&d, &kind, &absent, &ok_count};
+      e = cudaLaunchCooperativeKernel((const void*)wait_selftest_kernel, dim3(nblk), dim3(32), args, 0, s);
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h[0], &d.res->timeout, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h[1], ok_count, 4, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    timed_out += h[0] != 0;
+    passed += h[1];
+    // with a block missing no block may pass and every wait must run out; with none missing the reverse
+    if ((absent ? h[0] == 0 || h[1] != 0 : h[0] != 0 || h[1] != nblk) && wrong < 0) wrong = kind;
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h[0], timeout, 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h[1], ok_count, 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(buf);
   if (e != cudaSuccess) return cuda_fail(e, "cgp_barrier_selftest");
-  if (h[0]) return fail(CGP_ERR_TIMEOUT, "cgp_barrier_selftest: barrier timed out (" + std::to_string(h[1]) +
-                                             " blocks passed)");
-  if (h[1] != nblk - absent) return fail(CGP_ERR_CUDA, "cgp_barrier_selftest: blocks missing without timeout");
+  if (wrong >= 0 && absent) return fail(CGP_ERR_CUDA, "cgp_barrier_selftest: blocks missing without timeout (wait " + std::to_string(wrong) + ")");
+  if (wrong >= 0 && !timed_out) return fail(CGP_ERR_CUDA, "cgp_barrier_selftest: wrong values (wait " + std::to_string(wrong) + ")");
+  if (timed_out) return fail(CGP_ERR_TIMEOUT, "cgp_barrier_selftest: waits timed out (" + std::to_string(passed) + " blocks passed)");
   return CGP_OK;
 }
 
