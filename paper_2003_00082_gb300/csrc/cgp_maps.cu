@@ -255,20 +255,33 @@ __global__ void correct_fill_kernel(int n_f, const int* __restrict__ ptr, const 
   col[at] = i;
   coef[at] = make_double2(ox * ia, oy * ia);
   at += 32;
-  const bool merge = e1 - e0 <= kMergeEntries;
-  for (int e = e0; e < e1; ++e) {
-    if (merge && !first_seen(ent, e0, e)) continue;
-    double wx = 0.0, wy = 0.0;
-    for (int f = merge ? e0 : e; f < (merge ? e1 : e + 1); ++f) {
-      if (ent[f] != ent[e]) continue;
-      const bool second = (f - e0) & 1;   // this neighbour is k of (i, j, k), else j
-      const double2 xo = xy[ent[second ? f - 1 : f + 1]];
-      wx += second ? xi.y - xo.y : xo.y - xi.y;
-      wy += second ? xo.x - xi.x : xi.x - xo.x;
+  if (e1 - e0 > kMergeEntries) {
+#pragma unroll 8
+    for (int e = e0; e < e1; e += 2) {   // a hub, triangle by triangle: independent loads in flight
+      const int j = ent[e], k = ent[e + 1];
+      const double2 xj = xy[j], xk = xy[k];
+      const long long q = at + 32LL * (e - e0);
+      col[q] = j;
+      coef[q] = make_double2((xk.y - xi.y) * ia, (xi.x - xk.x) * ia);
+      col[q + 32] = k;
+      coef[q + 32] = make_double2((xi.y - xj.y) * ia, (xj.x - xi.x) * ia);
     }
-    col[at] = ent[e];
-    coef[at] = make_double2(wx * ia, wy * ia);
-    at += 32;
+    at += 32LL * (e1 - e0);
+  } else {
+    for (int e = e0; e < e1; ++e) {
+      if (!first_seen(ent, e0, e)) continue;
+      double wx = 0.0, wy = 0.0;
+      for (int f = e0; f < e1; ++f) {
+        if (ent[f] != ent[e]) continue;
+        const bool second = (f - e0) & 1;   // this neighbour is k of (i, j, k), else j
+        const double2 xo = xy[ent[second ? f - 1 : f + 1]];
+        wx += second ? xi.y - xo.y : xo.y - xi.y;
+        wy += second ? xo.x - xi.x : xi.x - xo.x;
+      }
+      col[at] = ent[e];
+      coef[at] = make_double2(wx * ia, wy * ia);
+      at += 32;
+    }
   }
   for (; at < end; at += 32) {
     col[at] = i;
