@@ -972,7 +972,6 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
 
   // register rows: the first NE entries (absent ones: value 0 at the row's own
   // position) and whether a row goes on after them
-  constexpr bool VREG = R == 1 || R == 2;            // u_(k-1) in registers too
   float rq[NR], sq[NR], wq[NR], uq[NR], vq[NR], dq[NR], aq[NR][NE];
   unsigned cq[NR][NE / 2];
   unsigned out = 0, more = 0;                        // rows to publish; rows longer than NE
@@ -1105,11 +1104,11 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
       if (k > 0) {
         const float alpha = fs.abf[(k - 1) & 1][0], beta = fs.abf[(k - 1) & 1][1];
         own_rows([&](int q, int i) {
-          const float uo = VREG ? vq[q] : iu[i];
+          const float uo = R > 0 ? vq[q] : iu[i];   // u_(k-1)
           const float pi = k == 1 ? uo : fmaf(beta, ip[i], uo);
           ip[i] = pi;
           ie[i] = fmaf(alpha, pi, ie[i]);
-          if (!VREG) iu[i] = R > 0 ? uq[q] : ext[i];
+          if constexpr (R == 0) iu[i] = ext[i];
         });
       }
       // ---- the halo's w, then the sums ----
@@ -1137,7 +1136,7 @@ __device__ void solve_mixed_flow(const Desc& d, int lb, Shared& sh) {
         if constexpr (R > 0) {
           sq[q] = si;
           rq[q] = ri;
-          if (VREG) vq[q] = uq[q];
+          vq[q] = uq[q];
           uq[q] = ui;
         } else {
           is[i] = si;
