@@ -64,8 +64,8 @@ def workload_config(precision="fp64"):
 # (the bench's launch shape).  They hold only for the kernel sources they were
 # taken on and for the captured launch's tuning flags: when the sources' hash
 # or the benchmarked flags differ the traffic is reported as null.
-SOLVER_SOURCES = ("cgp_pcg.cu", "cgp_pcg_batch.cu", "cgp_pipe.cu", "cgp_solver.cuh", "cgp_sync.h", "cgp_fixed.h",
-                  "cgp_internal.h")
+SOLVER_SOURCES = ("cgp_pcg.cu", "cgp_pcg_batch.cu", "cgp_pipe.cu", "cgp_flow.cu", "cgp_flow.cuh", "cgp_solver.cuh",
+                  "cgp_sync.h", "cgp_fixed.h", "cgp_internal.h")
 SOLVER_TRAFFIC = {
     "sha256": "bd624dbe15e1ef9e4fd16d5f924229b690a886bbac437062f633aa27336c60dd",
     "fp64": 10377984 + 335616,
