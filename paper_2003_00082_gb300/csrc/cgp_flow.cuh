@@ -33,8 +33,8 @@
 // apart (the pollers queue on the shared lines), 3.5k through slots on lines
 // of their own stored with release, 2.6k stored relaxed; a line read on the
 // other die just after it was written costs about 1.7k of that.  Polling loads
-// the same network that the words travel on, so a round has one lane and one
-// load per block.  The rest of an iteration is a chain of short steps (warp
+// the same network that the words travel on, so a round has one lane a block and
+// one load a word.  The rest of an iteration is a chain of short steps (warp
 // sums, block sums, totals, scalars), each written for latency here.
 #pragma once
 
@@ -181,8 +181,8 @@ __device__ __forceinline__ void flow_rows(const int* __restrict__ row, const int
 
 // The sums are those of put_partials (cgp_fixed.h): 128-bit integers aligned to
 // the largest exponent, value X 2^(E - 1129).  A block's sum travels in one word
-// (fx::pack_word: 94 bits below its largest term; two words with all of X cost
-// 4300 clocks an iteration on 152 blocks, since polling loads the network), and
+// (fx::pack_word: 94 bits below its largest term; two words with all of X took
+// 3700 clocks more of an iteration on 152 blocks, since polling loads the network), and
 // the fold over the blocks is 128 bits wide again.  A warp's sum is five
 // redux.sync of 27-bit limbs.  Sums of 57-bit images, truncated 2^-54 below the
 // largest term of a warp, block or group, took 7 % less of a solve at 512x256 and
@@ -409,7 +409,7 @@ __device__ __forceinline__ bool flow_fetch64(const Desc& d, int red, const int* 
 //
 // Measured at 512x256 on 152 blocks in O-grid tiles: 6.83 us an iteration with
 // the counter barrier and slots 16 bytes apart, 6.34 us with all sums after the
-// product, 5.59 us in this form.
+// product, 5.59 us in this form with 57-bit images, 5.9 us with 128-bit ones.
 constexpr int kFlowMinBlock = 256;
 template <int T>
 __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
@@ -423,11 +423,12 @@ __device__ void solve_fp64_flow(const Desc& d, int lb, Shared& sh) {
   const int ow = nw / 2, ct = 32 * ow;                  // warps and threads with rows
   const int act = min(ow, (nloc * T + 31) / 32);        // of those, warps that have any
   const int G = flow_groups(d.nblk, nw - ow - 2);       // warps ow .. ow + G - 1 poll, warp ow + G derives the scalars
-  // With many rows the product outlasts the early words by far: the warps that
-  // poll for what it gives wait until this block's own part is done (866 rows:
-  // 5.72 -> 5.59 us an iteration, 745 rows: 6.98 -> 6.75 ms a solve).  With few
-  // rows the words are there almost at once and the wait costs a round trip (95
-  // rows: 1.23 -> 1.34 ms, 346 rows: 3.73 -> 3.81 ms).
+  // With many rows the product outlasts the early words: the warps that poll for
+  // what it gives wait until this block's own part is done.  In the bisection
+  // order this pays from about 500 rows a block (a solve with 429 rows: 5.06 ms
+  // without, 5.11 with; 529 rows: 6.54 and 6.40; 866 rows: 9.86 and 9.75), on
+  // O-grid tiles, whose product is shorter, from about 850 (583 rows: 6.37 and
+  // 6.51; 866 rows: 8.85 and 8.75); with few rows the wait costs a round trip.
   const bool patient = chunk >= 512;
   double* const R0 = d.pub64 + 4 * n;                // r of a pass's start, for the ghost rows
   int* const mark = reinterpret_cast<int*>(d.z);     // rows that another block reads

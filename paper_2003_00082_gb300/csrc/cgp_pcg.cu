@@ -743,22 +743,25 @@ void free_perm_system(PermSystem& ps) {
 // shape used).  The dataflow iterations (flag bit 3) wherever rows fit in shared
 // memory, 512 threads a block.  FP64: about 96 rows a block, since the exchange
 // costs nearly the same for any number of blocks while the FP64 pipe of every SM
-// takes its share of the rows (129x67: 1.24 ms on 92 blocks, 1.47 ms on 24);
-// O-grid tiles where the mesh is registered (512x256: 7.4 ms against 8.2 ms in the
-// bisection order and 10.2 ms in the mesh's own), else the bisection order from
-// 4096 rows on (321x163: 3.7 against 4.1 ms), below which it gains nothing.
+// takes its share of the rows (129x67: 1.51 ms on 92 blocks, 1.56 on 138, 1.86 on
+// 25; between 2700 and 6200 rows 64 rows a block are still 3 to 8 % faster: 74x36
+// 0.83 against 0.86 ms, 110x55 1.25 against 1.30); O-grid tiles where the mesh is
+// registered (512x256: 8.8 ms against 9.7 ms in the bisection order and 11.6 ms in
+// the mesh's own), else the bisection order from 4096 rows on (321x163: 4.5
+// against 4.8 ms), below which it gains under 1 %.
 // MIXED: about 352 rows a block but at least 12 blocks, in the mesh's order: up to
-// about 12 blocks share one GPC, where the exchange is shortest (90x45: 0.60 ms on
-// 12 blocks, 0.69 ms on 17); bisection gains under 1 % at any size and costs a
+// about 12 blocks share one GPC, where the exchange is shortest (64x32: 0.58 ms on
+// 12 blocks of 256 threads, 0.62 on 6 of them or 17 of 512); bisection gains about 1 % at any size and costs a
 // second copy of the system.  Below 2500 rows a block has 256 threads, whose
-// barriers are cheaper (64x32: FP64 0.545 ms on 33 blocks of 256 threads, 0.567 ms
-// on 22 of 512; MIXED 0.42 and 0.44 ms on 12).  Systems whose rows do not fit keep
-// the barrier forms with rows in global memory; so does a solve under stream
-// capture whose renumbered system or halo lists are not there yet, since building
-// them allocates and synchronises.  A form that does not fit, or whose system
-// cannot be allocated, is no reason to refuse the solve: the next one is taken,
-// and the mesh remembers it, so that later solves do not try (and synchronise)
-// again.
+// barriers are cheaper, and in FP64 64 rows (64x32: FP64 0.69 ms on 33 blocks of
+// 256 threads, 0.72 of 512, 0.74 on 22; MIXED on 12 blocks 0.58 and 0.61 ms; at
+// 3280 rows the order has turned, MIXED 0.85 and 0.80).  Times at tol 1e-10 from
+// x = 0.  Systems whose rows do not fit keep the barrier forms with rows in global
+// memory; so does a solve under stream capture whose renumbered system or halo
+// lists are not there yet, since building them allocates and synchronises.  A form
+// that does not fit, or whose system cannot be allocated, is no reason to refuse
+// the solve: the next one is taken, and the mesh remembers it, so that later
+// solves do not try (and synchronise) again.
 int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps, SolverTuning& tu, cudaStream_t s) {
   const int n = m->n_c, sms = std::max(1, dev_info(m->device).sms);
   const bool small = n < 2500;
