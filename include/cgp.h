@@ -281,7 +281,8 @@ int cgp_poisson_solve_noalloc(int n, const int* rowptr, const int* col, const do
  *                     cgp_set_tuning; bits 5-6: waves
  *                     with 256 << k rows per block).  INVALID_ARG for other
  *                     bits.  All zero (as after cgp_batch_create): waves with
- *                     tagged reductions where rows fit in shared memory.
+ *                     bit 3's iterations without a grid barrier where they fit
+ *                     in shared memory, untagged reductions elsewhere.
  * cgp_batch_autotune  times a set of launch shapes on the batch's own
  *                     systems (from x = 0) and keeps the fastest; writes the
  *                     best time in ms to best_ms (nullable).  Synchronous;
@@ -477,8 +478,9 @@ int cgp_mesh_set_ogrid(cgp_mesh m, int n_theta, int n_r);
  *         try this form); other bits must be 0.
  *         SpMV: bit 0 uses the O-grid stencil form (cgp_mesh_set_ogrid) with
  *         one thread per row (lanes ignored).
- * All zero (as after cgp_assemble) lets the solver choose: tagged reductions
- * with rows in shared memory where they fit; FP64 about 96 rows per block (64
+ * All zero (as after cgp_assemble) lets the solver choose: bit 3's iterations
+ * without a grid barrier where they fit in shared memory (else the untagged
+ * single-reduction form); FP64 about 96 rows per block (64
  * below 2500 rows), on O-grid tiles (registered meshes) or, from 4096 rows on,
  * in the bisection order (the renumbered system is built by the first solve);
  * MIXED about 352 rows per block on at least 12 blocks.

@@ -761,7 +761,9 @@ void free_perm_system(PermSystem& ps) {
 // lists are not there yet, since building them allocates and synchronises.  A form
 // that does not fit, or whose system cannot be allocated, is no reason to refuse
 // the solve: the next one is taken, and the mesh remembers it, so that later
-// solves do not try (and synchronise) again.
+// solves do not try (and synchronise) again.  Without the dataflow iterations the
+// sums stay the exact ones of the untagged form: the barrier's tagged sums are for
+// callers who ask for them.
 int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps, SolverTuning& tu, cudaStream_t s) {
   const int n = m->n_c, sms = std::max(1, dev_info(m->device).sms);
   const bool small = n < 2500;
@@ -794,7 +796,7 @@ int plan_default(cgp_mesh_impl* m, bool mixed, LaunchPlan& out, PermSystem** ps,
     const size_t systems = m->psys.size();
     if (built(flags[k]) || !(flags[k] & 36) || renumbered_rows_can_fit(m, nblk, block, (flags[k] & 32) != 0)) {
       tu = SolverTuning{block, 1, nblk, flags[k]};
-      if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.res) return CGP_OK;
+      if (plan_solve(m, m->device, n, m->max_blocks, tu, mixed, out, ps) == CGP_OK && out.flow) return CGP_OK;
     }
     if (m->psys.size() > systems) {   // built here, and its halo was too much
       free_perm_system(m->psys.back());
@@ -1264,7 +1266,7 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
   const int lanes = sh.lanes > 0 ? sh.lanes : 1;
   const int block = sh.block > 0 ? sh.block : 512;
   const bool mixed = o.precision == CGP_MIXED;
-  // never tuned: tagged reductions (dataflow iterations) where a wave's rows are resident
+  // never tuned: dataflow iterations where a wave's rows leave room for them, else untagged reductions
   const bool untuned = sh.block == 0 && sh.lanes == 0 && sh.per_sm == 0 && sh.flags == 0;
   const int flags = untuned ? 8 : sh.flags;
   BatchFn fn0 = batched_kernel_for(lanes, false);
@@ -1381,7 +1383,7 @@ int batch_plan_waves(cgp_batch_s* B, const BatchShape& sh, const cgp_solve_opts&
       }
       unsigned char* ctrl = B->d_ctrl + kCtrlPerInstance * i;
       desc[i] = make_desc(m, B->b[i], B->x[i], o, nb[i], lp, reinterpret_cast<unsigned*>(ctrl),
-                          reinterpret_cast<SolveResult*>(ctrl + 256), untuned && !res ? 0 : flags);
+                          reinterpret_cast<SolveResult*>(ctrl + 256), untuned && !rl.flow ? 0 : flags);
       desc[i].blk0 = blk0;
       if (max_epochs(o) * nb[i] >= (1LL << 31)) return fail(CGP_ERR_INVALID_ARG, "batch: max_it too large");
       for (int k = 0; k < nb[i]; ++k) blk_inst.push_back(i);
