@@ -67,8 +67,8 @@ def workload_config(precision="fp64"):
 SOLVER_SOURCES = ("cgp_pcg.cu", "cgp_pcg_batch.cu", "cgp_pipe.cu", "cgp_flow.cu", "cgp_flow.cuh", "cgp_solver.cuh",
                   "cgp_sync.h", "cgp_fixed.h", "cgp_internal.h")
 SOLVER_TRAFFIC = {
-    "sha256": "bd624dbe15e1ef9e4fd16d5f924229b690a886bbac437062f633aa27336c60dd",
-    "fp64": 10377984 + 335616,
+    "sha256": "5ccd1f3117f4f5e1c1d5e5cfd5e46e3170020aa539dc5c8f101f64d8525db853",
+    "fp64": 10485248 + 94976,
     "flags": {"fp64": 40},
 }
 

@@ -103,8 +103,8 @@ struct ForceCoef {
 // kept per parent since assembly (parent_shape_kernel), give a gradient in four
 // operations, and the middle child's differences are two of the others'.
 //
-// The FP64 pipe bounds it (16 clocks a warp operation and SM): 22 operations a
-// parent for the gradients and 38 for the force, against 51 and 38 when each
+// The FP64 pipe bounds it (16 clocks a warp operation and SM): 20 operations a
+// parent for the gradients and 38 for the force, against 50 and 38 when each
 // launch formed the geometry and a division.  512x256 (262,144 parents): 48.4 -> 34.3 us
 // with the force, 29.5 -> 15.0 us without (25 and 10 us of FP64 pipe).
 template <bool FORCE>
