@@ -282,6 +282,7 @@ int get_perm_system(cgp_mesh_impl* m, int nblk, PermSystem*& out, int tiles = 0)
   const int n = m->n_c, nnz = m->nnz, chunk = (n + nblk - 1) / nblk;
   const double* const K = dir ? m->Kd : m->K;
   std::vector<Point> pts(n);
+  CGP_CUDA(cudaDeviceSynchronize());
   if (tiles) {
     for (int j = 0, i = 0; i < n; ++j)   // (angle index, ring index)
       for (int t = 0; t < m->st_nt; ++t, ++i) pts[i] = Point{{(double)t, (double)j}, i};
@@ -305,9 +306,21 @@ int get_perm_system(cgp_mesh_impl* m, int nblk, PermSystem*& out, int tiles = 0)
   ps.h_rowptr.assign(n + 1, 0);
   ps.h_col.resize(nnz);
   std::vector<int> src(nnz);   // the mesh's entry of every entry
+  std::vector<std::pair<int, int>> hub;
   for (int r = 0; r < n; ++r) {
     const int o = perm[r], k0 = ps.h_rowptr[r];
     int k1 = k0;
+    if (m->h_rowptr[o + 1] - m->h_rowptr[o] > 32) {   // a hub
+      hub.clear();
+      for (int k = m->h_rowptr[o]; k < m->h_rowptr[o + 1]; ++k) hub.push_back({inv[m->h_col[k]], k});
+      std::sort(hub.begin(), hub.end());
+      for (const auto& e : hub) {
+        ps.h_col[k1] = e.first;
+        src[k1++] = e.second;
+      }
+      ps.h_rowptr[r + 1] = k1;
+      continue;
+    }
     for (int k = m->h_rowptr[o]; k < m->h_rowptr[o + 1]; ++k, ++k1) {   // few entries a row: insertion sort
       const int c = inv[m->h_col[k]];
       int q = k1;
