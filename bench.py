@@ -67,8 +67,8 @@ def workload_config(precision="fp64"):
 SOLVER_SOURCES = ("cgp_pcg.cu", "cgp_pcg_batch.cu", "cgp_pipe.cu", "cgp_flow.cu", "cgp_flow.cuh", "cgp_solver.cuh",
                   "cgp_sync.h", "cgp_fixed.h", "cgp_internal.h")
 SOLVER_TRAFFIC = {
-    "sha256": "5ccd1f3117f4f5e1c1d5e5cfd5e46e3170020aa539dc5c8f101f64d8525db853",
-    "fp64": 10485248 + 94976,
+    "sha256": "4277f034b626773f37807ae5b9c178e94b23a88e9bc03eb425d7e07be13c5ee0",
+    "fp64": 10422016 + 97280,
     "flags": {"fp64": 40},
 }
 
